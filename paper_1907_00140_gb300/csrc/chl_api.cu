@@ -91,6 +91,67 @@ int device_sms() {
 
 namespace {
 
+// Host-mapped staging of the query calls: the kernel sets its bad-vertex flag
+// in it, and a batch of up to STAGE_PAIRS host pairs is read from it and
+// answered into it, so that such a call is one launch and one wait (an
+// allocation, a memset and up to three copies before: one pair 44 us, now 21).
+// A call takes a block and gives it back before it returns, so blocks are never
+// shared between threads or streams; at most STAGE_BLOCKS exist, of which
+// STAGE_IDLE stay allocated while no call uses them. A call that gets none
+// takes the general path.
+constexpr uint64_t STAGE_PAIRS = 4096;
+constexpr int STAGE_BLOCKS = 8, STAGE_IDLE = 2;
+
+struct StageBlock {
+    uint32_t pairs[2 * STAGE_PAIRS];
+    uint32_t out[STAGE_PAIRS];
+    int bad;
+};
+
+struct Stage {
+    StageBlock *b = nullptr;
+    static std::mutex mu;
+    static StageBlock *idle[STAGE_IDLE];
+    static int n_idle, made;
+    Stage() {
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            if (n_idle) b = idle[--n_idle];
+            else if (made < STAGE_BLOCKS) ++made;
+            else return;
+        }
+        if (!b) {
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, sizeof(StageBlock), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+                b = static_cast<StageBlock *>(p);
+            } else {
+                (void)cudaGetLastError();
+                std::lock_guard<std::mutex> lk(mu);
+                --made;
+                return;
+            }
+        }
+        b->bad = 0;
+    }
+    ~Stage() {
+        if (!b) return;
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            if (n_idle < STAGE_IDLE) {
+                idle[n_idle++] = b;
+                return;
+            }
+            --made;
+        }
+        cudaFreeHost(b);
+    }
+    Stage(const Stage &) = delete;
+    Stage &operator=(const Stage &) = delete;
+};
+std::mutex Stage::mu;
+StageBlock *Stage::idle[STAGE_IDLE] = {};
+int Stage::n_idle = 0, Stage::made = 0;
+
 // device control block of one tree launch; the two counters every tree
 // updates sit on cache lines of their own
 struct Control {
@@ -1220,56 +1281,67 @@ extern "C" chl_status chl_query(const chl_labels *L, const uint32_t *pairs, uint
     b_p.s = b_o.s = b_bad.s = s;
     const uint32_t *dp = pairs;
     uint32_t *dout = out;
-    int hbad = 0;
-    CUDA_TRY(dmalloc(&b_bad.p, sizeof(int), s));
-    CUDA_TRY(cudaMemsetAsync(b_bad.p, 0, sizeof(int), s));
-    if (mem == CHL_MEM_HOST) {
+    int hbad = 0, *bad = nullptr;
+    Stage stage;
+    const bool staged = stage.b && mem == CHL_MEM_HOST && q <= STAGE_PAIRS;
+    if (stage.b) {
+        bad = &stage.b->bad;
+    } else {
+        CUDA_TRY(dmalloc(&b_bad.p, sizeof(int), s));
+        CUDA_TRY(cudaMemsetAsync(b_bad.p, 0, sizeof(int), s));
+        bad = (int *)b_bad.p;
+    }
+    if (staged) {
+        std::memcpy(stage.b->pairs, pairs, q * 8);
+        dp = stage.b->pairs;
+        dout = stage.b->out;
+    } else if (mem == CHL_MEM_HOST) {
         CUDA_TRY(dmalloc(&b_p.p, q * 8, s));
         CUDA_TRY(dmalloc(&b_o.p, q * 4, s));
         CUDA_TRY(cudaMemcpyAsync(b_p.p, pairs, q * 8, cudaMemcpyHostToDevice, s));
         dp = (const uint32_t *)b_p.p;
         dout = (uint32_t *)b_o.p;
     }
-    CUDA_TRY(launch_query(L->n, L->offsets, L->hubpos, L->dist, dp, q, dout, (int *)b_bad.p, s));
-    if (mem == CHL_MEM_HOST) CUDA_TRY(cudaMemcpyAsync(out, dout, q * 4, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaMemcpyAsync(&hbad, b_bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(launch_query(L->n, L->offsets, L->hubpos, L->dist, dp, q, dout, bad, s));
+    if (mem == CHL_MEM_HOST && !staged) CUDA_TRY(cudaMemcpyAsync(out, dout, q * 4, cudaMemcpyDeviceToHost, s));
+    if (!stage.b) CUDA_TRY(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
+    if (staged) std::memcpy(out, stage.b->out, q * 4);
+    if (stage.b) hbad = stage.b->bad;
     if (hbad) st = set_error(CHL_EINVAL, "a query vertex id is >= n");
 done:
+    // a call that failed midway may have a kernel writing to its block
+    if (st == CHL_ECUDA || st == CHL_ENOMEM) cudaStreamSynchronize(s);
     return st;
 }
 
 // ------------------------------------------------------------------ query modes
 namespace {
 
-// a batch over one set (plain or partitioned) through the multi-set kernel:
-// device pairs and answers, the set descriptor and a flag in device memory
-chl_status run_set_query(const QuerySet &set, const QuerySet *parts_h, uint32_t nparts,
-                         const uint32_t *pairs, uint64_t q, uint32_t *out, chl_mem mem, bool grouped,
-                         cudaStream_t s) {
+// a batch over the lists of L in grouped order, or (nparts > 0) over hub
+// partitions in arrival order; the sets travel as kernel parameters
+chl_status run_mode_query(const QueryParts &sets, const uint32_t *pairs, uint64_t q, uint32_t *out, chl_mem mem,
+                          bool grouped, cudaStream_t s) {
     chl_status st = CHL_OK;
-    DevBuf b_set, b_p, b_o, b_perm, b_scr;
-    b_set.s = b_p.s = b_o.s = b_perm.s = b_scr.s = s;
+    DevBuf b_p, b_o, b_perm, b_scr, b_bad;
+    b_p.s = b_o.s = b_perm.s = b_scr.s = b_bad.s = s;
     const uint32_t *dp = pairs;
     uint32_t *dout = out;
-    int hbad = 0;
-    // [set][nsets, bad][parts]
-    const size_t hdr = sizeof(QuerySet) + 16;
-    std::vector<uint8_t> host(hdr + size_t(nparts) * sizeof(QuerySet));
-    QuerySet top = set;
-    uint8_t *base = nullptr;
-    CUDA_TRY(dmalloc(&b_set.p, host.size(), s));
-    base = static_cast<uint8_t *>(b_set.p);
-    if (nparts) top.parts = reinterpret_cast<const QuerySet *>(base + hdr);
-    std::memcpy(host.data(), &top, sizeof(QuerySet));
-    {
-        const uint32_t one = 1, zero = 0;
-        std::memcpy(host.data() + sizeof(QuerySet), &one, 4);
-        std::memcpy(host.data() + sizeof(QuerySet) + 4, &zero, 4);
+    int hbad = 0, *bad = nullptr;
+    Stage stage;
+    const bool staged = stage.b && mem == CHL_MEM_HOST && q <= STAGE_PAIRS;
+    if (stage.b) {
+        bad = &stage.b->bad;
+    } else {
+        CUDA_TRY(dmalloc(&b_bad.p, sizeof(int), s));
+        CUDA_TRY(cudaMemsetAsync(b_bad.p, 0, sizeof(int), s));
+        bad = (int *)b_bad.p;
     }
-    if (nparts) std::memcpy(host.data() + hdr, parts_h, size_t(nparts) * sizeof(QuerySet));
-    CUDA_TRY(cudaMemcpyAsync(base, host.data(), host.size(), cudaMemcpyHostToDevice, s));
-    if (mem == CHL_MEM_HOST) {
+    if (staged) {
+        std::memcpy(stage.b->pairs, pairs, q * 8);
+        dp = stage.b->pairs;
+        dout = stage.b->out;
+    } else if (mem == CHL_MEM_HOST) {
         CUDA_TRY(dmalloc(&b_p.p, q * 8, s));
         CUDA_TRY(dmalloc(&b_o.p, q * 4, s));
         CUDA_TRY(cudaMemcpyAsync(b_p.p, pairs, q * 8, cudaMemcpyHostToDevice, s));
@@ -1279,19 +1351,18 @@ chl_status run_set_query(const QuerySet &set, const QuerySet *parts_h, uint32_t 
     if (grouped) {
         CUDA_TRY(dmalloc(&b_perm.p, q * 4, s));
         CUDA_TRY(dmalloc(&b_scr.p, GROUP_SCRATCH_WORDS * 4, s));
-        CUDA_TRY(launch_group_order(reinterpret_cast<const QuerySet *>(base),
-                                    reinterpret_cast<const uint32_t *>(base + sizeof(QuerySet)), dp,
-                                    nullptr, q, (uint32_t *)b_scr.p, (uint32_t *)b_perm.p, s));
+        CUDA_TRY(launch_group_order_one(sets.n, dp, q, (uint32_t *)b_scr.p, (uint32_t *)b_perm.p, s));
     }
-    CUDA_TRY(launch_query_sets(reinterpret_cast<const QuerySet *>(base),
-                               reinterpret_cast<const uint32_t *>(base + sizeof(QuerySet)), dp, nullptr,
-                               grouped ? (const uint32_t *)b_perm.p : nullptr, q, dout,
-                               reinterpret_cast<int *>(base + sizeof(QuerySet) + 4), device_sms() * 64, s));
-    if (mem == CHL_MEM_HOST) CUDA_TRY(cudaMemcpyAsync(out, dout, q * 4, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaMemcpyAsync(&hbad, base + sizeof(QuerySet) + 4, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(launch_query_parts(sets, dp, grouped ? (const uint32_t *)b_perm.p : nullptr, q, dout, bad, s));
+    if (mem == CHL_MEM_HOST && !staged) CUDA_TRY(cudaMemcpyAsync(out, dout, q * 4, cudaMemcpyDeviceToHost, s));
+    if (!stage.b) CUDA_TRY(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
+    if (staged) std::memcpy(out, stage.b->out, q * 4);
+    if (stage.b) hbad = stage.b->bad;
     if (hbad) st = set_error(CHL_EINVAL, "a query vertex id is >= n");
 done:
+    // a call that failed midway may have a kernel writing to its block
+    if (st == CHL_ECUDA || st == CHL_ENOMEM) cudaStreamSynchronize(s);
     return st;
 }
 
@@ -1304,18 +1375,19 @@ extern "C" chl_status chl_query_partitioned(const chl_labels *const *parts, uint
     if (!parts) return set_error(CHL_EINVAL, "parts is NULL");
     if (nparts < 1 || nparts > CHL_MAX_PARTS)
         return set_error(CHL_EINVAL, "nparts must be in [1, %d]", CHL_MAX_PARTS);
-    std::vector<QuerySet> h(nparts);
+    QueryParts h;
+    h.nparts = nparts;
     for (uint32_t k = 0; k < nparts; ++k) {
         if (!parts[k]) return set_error(CHL_EINVAL, "part %u is NULL", k);
         CHECK_DEVICE(parts[k]);
         if (parts[k]->n != parts[0]->n) return set_error(CHL_EINVAL, "parts cover different vertex counts");
-        h[k] = QuerySet{parts[k]->n, parts[k]->offsets, parts[k]->hubpos, parts[k]->dist, 0, nullptr};
+        h.lists[k] = QueryLists{parts[k]->offsets, parts[k]->hubpos, parts[k]->dist};
     }
+    h.n = parts[0]->n;
     if (q == 0) return CHL_OK;
     if (!pairs || !out) return set_error(CHL_EINVAL, "pairs or out is NULL");
     if (mem != CHL_MEM_DEVICE && mem != CHL_MEM_HOST) return set_error(CHL_EINVAL, "unknown memory kind");
-    const QuerySet set{parts[0]->n, nullptr, nullptr, nullptr, nparts, nullptr};
-    return run_set_query(set, h.data(), nparts, pairs, q, out, mem, false, (cudaStream_t)stream);
+    return run_mode_query(h, pairs, q, out, mem, false, (cudaStream_t)stream);
 }
 
 extern "C" chl_status chl_query_grouped(const chl_labels *L, const uint32_t *pairs, uint64_t q,
@@ -1327,8 +1399,11 @@ extern "C" chl_status chl_query_grouped(const chl_labels *L, const uint32_t *pai
     if (!pairs || !out) return set_error(CHL_EINVAL, "pairs or out is NULL");
     if (mem != CHL_MEM_DEVICE && mem != CHL_MEM_HOST) return set_error(CHL_EINVAL, "unknown memory kind");
     if (q > 0xFFFFFFFFull) return set_error(CHL_EINVAL, "chl_query_grouped takes fewer than 2^32 pairs");
-    const QuerySet set{L->n, L->offsets, L->hubpos, L->dist, 0, nullptr};
-    return run_set_query(set, nullptr, 0, pairs, q, out, mem, true, (cudaStream_t)stream);
+    QueryParts h;
+    h.n = L->n;
+    h.nparts = 1;
+    h.lists[0] = QueryLists{L->offsets, L->hubpos, L->dist};
+    return run_mode_query(h, pairs, q, out, mem, true, (cudaStream_t)stream);
 }
 
 extern "C" void chl_labels_free(chl_labels *L) {
@@ -1379,9 +1454,15 @@ extern "C" chl_status chl_path(const chl_labels *L, const uint32_t *pairs, uint6
     b_p.s = b_path.s = b_len.s = b_bad.s = s;
     const uint32_t *dp = pairs;
     uint32_t *dpath = paths, *dlen = lens;
-    int hbad = 0;
-    CUDA_TRY(dmalloc(&b_bad.p, sizeof(int), s));
-    CUDA_TRY(cudaMemsetAsync(b_bad.p, 0, sizeof(int), s));
+    int hbad = 0, *bad = nullptr;
+    Stage stage;
+    if (stage.b) {
+        bad = &stage.b->bad;
+    } else {
+        CUDA_TRY(dmalloc(&b_bad.p, sizeof(int), s));
+        CUDA_TRY(cudaMemsetAsync(b_bad.p, 0, sizeof(int), s));
+        bad = (int *)b_bad.p;
+    }
     if (mem == CHL_MEM_HOST) {
         CUDA_TRY(dmalloc(&b_p.p, q * 8, s));
         CUDA_TRY(dmalloc(&b_path.p, q * max_len * 4 + 4, s));
@@ -1392,16 +1473,19 @@ extern "C" chl_status chl_path(const chl_labels *L, const uint32_t *pairs, uint6
         dlen = (uint32_t *)b_len.p;
     }
     CUDA_TRY(launch_paths(L->n, L->offsets, L->hubpos, L->dist, L->hub, L->parent, dp, q, max_len,
-                          dpath, dlen, (int *)b_bad.p, s));
+                          dpath, dlen, bad, s));
     if (mem == CHL_MEM_HOST) {
         if (max_len) CUDA_TRY(cudaMemcpyAsync(paths, dpath, q * max_len * 4, cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaMemcpyAsync(lens, dlen, q * 4, cudaMemcpyDeviceToHost, s));
     }
-    CUDA_TRY(cudaMemcpyAsync(&hbad, b_bad.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    if (!stage.b) CUDA_TRY(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
+    if (stage.b) hbad = stage.b->bad;
     if (hbad == 1) st = set_error(CHL_EINVAL, "a query vertex id is >= n");
     else if (hbad) st = set_error(CHL_ECUDA, "a parent chain did not reach its hub");
 done:
+    // a call that failed midway may have a kernel writing to its block
+    if (st == CHL_ECUDA || st == CHL_ENOMEM) cudaStreamSynchronize(s);
     return st;
 }
 

@@ -195,6 +195,19 @@ struct QuerySet {
 cudaError_t launch_query_sets(const QuerySet *sets, const uint32_t *nsets, const uint32_t *pairs,
                               const uint16_t *set_of, const uint32_t *perm, uint64_t q, uint32_t *out,
                               int *bad, int max_blocks, cudaStream_t s);
+// the same answers for one set given as a kernel parameter: its lists, or its
+// hub partitions (the minimum over them); perm as above
+struct QueryLists {
+    const uint64_t *offsets;
+    const uint32_t *hubpos;
+    const uint32_t *dist;
+};
+struct QueryParts {
+    uint32_t n, nparts;
+    QueryLists lists[CHL_MAX_PARTS];
+};
+cudaError_t launch_query_parts(const QueryParts &sets, const uint32_t *pairs, const uint32_t *perm, uint64_t q,
+                               uint32_t *out, int *bad, cudaStream_t s);
 // grouped order of a batch: perm[0..q) = the pairs sorted by the block pair of
 // their two vertices (64 blocks per set); set_of may be null (all set 0);
 // scratch holds 4096 counters
@@ -202,6 +215,9 @@ constexpr uint32_t GROUP_SCRATCH_WORDS = 4096;
 cudaError_t launch_group_order(const QuerySet *sets, const uint32_t *nsets, const uint32_t *pairs,
                                const uint16_t *set_of, uint64_t q, uint32_t *scratch, uint32_t *perm,
                                cudaStream_t s);
+// ... of a batch over one set of n vertices
+cudaError_t launch_group_order_one(uint32_t n, const uint32_t *pairs, uint64_t q, uint32_t *scratch,
+                                   uint32_t *perm, cudaStream_t s);
 
 // exclusive prefix sum of n uint64 values (out may alias in); chl_graph.cu
 cudaError_t exclusive_scan_u64(const uint64_t *in, uint64_t *out, uint64_t n, cudaStream_t s,

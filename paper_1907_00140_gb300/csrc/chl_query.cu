@@ -432,6 +432,35 @@ __global__ void __launch_bounds__(QUERY_TPB, QUERY_CTAS) query_sets_kernel(const
     }
 }
 
+// a batch over one set, which travels as a kernel parameter
+__global__ void __launch_bounds__(QUERY_TPB, QUERY_CTAS)
+query_parts_kernel(const __grid_constant__ QueryParts sets, const uint32_t *__restrict__ pairs,
+                   const uint32_t *__restrict__ perm, uint64_t q, uint32_t *__restrict__ out, int *bad) {
+    __shared__ __align__(16) uint32_t tabs[QUERY_WARPS][TAB];
+    Table tab{tabs[threadIdx.x >> 5], 0};
+    table_clear(tab.slot);
+    const uint32_t lane = threadIdx.x & 31, each = pairs_per_warp(q);
+    const uint64_t warp = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
+    for (uint64_t j0 = warp * each; j0 < q; j0 += warps * each) {
+        const uint64_t j = j0 + lane;
+        const bool mine = lane < each && j < q;
+        uint64_t i = 0;
+        uint32_t u = 0, v = 0, d = 0xFFFFFFFFu;
+        if (mine) {
+            i = perm ? __ldg(&perm[j]) : j;
+            u = __ldg(&pairs[2 * i]);
+            v = __ldg(&pairs[2 * i + 1]);
+        }
+        const bool ok = mine && u < sets.n && v < sets.n;
+        if (mine && !ok) atomicExch(bad, 1);
+        const unsigned mask = __ballot_sync(FULL, ok);
+        for (uint32_t p = 0; p < sets.nparts; ++p)
+            merge_batch(sets.lists[p].offsets, sets.lists[p].hubpos, sets.lists[p].dist, mask, u, v, tab, d);
+        if (mine) out[i] = d;
+    }
+}
+
 // ---- grouped order (QDOL-style, Sec. 6: queries sorted and grouped by the
 // vertex partitions they touch, answers rearranged back into arrival order).
 // On one GPU a partition is a block of vertex ids: a pair's key is the block
@@ -443,12 +472,7 @@ __global__ void __launch_bounds__(QUERY_TPB, QUERY_CTAS) query_sets_kernel(const
 constexpr uint32_t GROUP_BLOCKS = 64;
 constexpr uint32_t GROUP_KEYS = GROUP_BLOCKS * GROUP_BLOCKS;
 
-__device__ __forceinline__ uint32_t group_key(const QuerySet *sets, uint32_t nsets, const uint32_t *pairs,
-                                              const uint16_t *set_of, uint64_t i) {
-    const uint32_t k = set_of ? __ldg(&set_of[i]) : 0;
-    if (k >= nsets) return 0;
-    const uint32_t n = sets[k].n;
-    uint32_t u = __ldg(&pairs[2 * i]), v = __ldg(&pairs[2 * i + 1]);
+__device__ __forceinline__ uint32_t group_key(uint32_t n, uint32_t u, uint32_t v) {
     if (u >= n || v >= n) return 0;
     if (u > v) {
         const uint32_t t = u;
@@ -459,12 +483,27 @@ __device__ __forceinline__ uint32_t group_key(const QuerySet *sets, uint32_t nse
     return bu * GROUP_BLOCKS + bv;
 }
 
-__global__ void group_count_kernel(const QuerySet *sets, const uint32_t *nsets_p, const uint32_t *pairs,
-                                   const uint16_t *set_of, uint64_t q, uint32_t *cnt) {
-    const uint32_t nsets = *nsets_p;
+// the set sizes of a batch: of its pairs' sets, or of its one set (sets null)
+struct GroupSets {
+    const QuerySet *sets;
+    const uint32_t *nsets;
+    const uint16_t *set_of;
+    uint32_t n;
+    __device__ __forceinline__ uint32_t key(const uint32_t *pairs, uint64_t i) const {
+        uint32_t size = n;
+        if (sets) {
+            const uint32_t k = set_of ? __ldg(&set_of[i]) : 0;
+            if (k >= *nsets) return 0;
+            size = sets[k].n;
+        }
+        return group_key(size, __ldg(&pairs[2 * i]), __ldg(&pairs[2 * i + 1]));
+    }
+};
+
+__global__ void group_count_kernel(GroupSets g, const uint32_t *pairs, uint64_t q, uint32_t *cnt) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < q;
          i += uint64_t(gridDim.x) * blockDim.x)
-        atomicAdd(&cnt[group_key(sets, nsets, pairs, set_of, i)], 1u);
+        atomicAdd(&cnt[g.key(pairs, i)], 1u);
 }
 
 // exclusive prefix of the GROUP_KEYS counts, in place (one CTA of 1024 threads)
@@ -504,12 +543,25 @@ __global__ void __launch_bounds__(1024) group_scan_kernel(uint32_t *cnt) {
     }
 }
 
-__global__ void group_scatter_kernel(const QuerySet *sets, const uint32_t *nsets_p, const uint32_t *pairs,
-                                     const uint16_t *set_of, uint64_t q, uint32_t *fill, uint32_t *perm) {
-    const uint32_t nsets = *nsets_p;
+__global__ void group_scatter_kernel(GroupSets g, const uint32_t *pairs, uint64_t q, uint32_t *fill,
+                                     uint32_t *perm) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < q;
          i += uint64_t(gridDim.x) * blockDim.x)
-        perm[atomicAdd(&fill[group_key(sets, nsets, pairs, set_of, i)], 1u)] = uint32_t(i);
+        perm[atomicAdd(&fill[g.key(pairs, i)], 1u)] = uint32_t(i);
+}
+
+cudaError_t group_order(const GroupSets &g, const uint32_t *pairs, uint64_t q, uint32_t *scratch, uint32_t *perm,
+                        cudaStream_t s) {
+    if (q == 0) return cudaSuccess;
+    if (q > 0xFFFFFFFFull) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(scratch, 0, GROUP_KEYS * sizeof(uint32_t), s);
+    if (e) return e;
+    uint64_t blocks = (q + 255) / 256;
+    if (blocks > uint64_t(device_sms()) * 8) blocks = uint64_t(device_sms()) * 8;
+    group_count_kernel<<<unsigned(blocks), 256, 0, s>>>(g, pairs, q, scratch);
+    group_scan_kernel<<<1, 1024, 0, s>>>(scratch);
+    group_scatter_kernel<<<unsigned(blocks), 256, 0, s>>>(g, pairs, q, scratch, perm);
+    return cudaGetLastError();
 }
 
 // a larger batch runs on as many CTAs as are resident at once, so that the
@@ -524,15 +576,19 @@ uint64_t resident_blocks(uint64_t blocks) {
 cudaError_t launch_group_order(const QuerySet *sets, const uint32_t *nsets, const uint32_t *pairs,
                                const uint16_t *set_of, uint64_t q, uint32_t *scratch, uint32_t *perm,
                                cudaStream_t s) {
+    return group_order(GroupSets{sets, nsets, set_of, 0}, pairs, q, scratch, perm, s);
+}
+
+cudaError_t launch_group_order_one(uint32_t n, const uint32_t *pairs, uint64_t q, uint32_t *scratch,
+                                   uint32_t *perm, cudaStream_t s) {
+    return group_order(GroupSets{nullptr, nullptr, nullptr, n}, pairs, q, scratch, perm, s);
+}
+
+cudaError_t launch_query_parts(const QueryParts &sets, const uint32_t *pairs, const uint32_t *perm, uint64_t q,
+                               uint32_t *out, int *bad, cudaStream_t s) {
     if (q == 0) return cudaSuccess;
-    if (q > 0xFFFFFFFFull) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(scratch, 0, GROUP_KEYS * sizeof(uint32_t), s);
-    if (e) return e;
-    uint64_t blocks = (q + 255) / 256;
-    if (blocks > uint64_t(device_sms()) * 8) blocks = uint64_t(device_sms()) * 8;
-    group_count_kernel<<<unsigned(blocks), 256, 0, s>>>(sets, nsets, pairs, set_of, q, scratch);
-    group_scan_kernel<<<1, 1024, 0, s>>>(scratch);
-    group_scatter_kernel<<<unsigned(blocks), 256, 0, s>>>(sets, nsets, pairs, set_of, q, scratch, perm);
+    const uint64_t blocks = resident_blocks((q * 32 + QUERY_TPB - 1) / QUERY_TPB);
+    query_parts_kernel<<<unsigned(blocks), QUERY_TPB, 0, s>>>(sets, pairs, perm, q, out, bad);
     return cudaGetLastError();
 }
 
