@@ -35,8 +35,9 @@ __all__ = [
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
-_SOURCES = ["chl_api.cu", "chl_graph.cu", "chl_tree.cu", "chl_labels.cu", "chl_query.cu",
+_SOURCES = ["chl_api.cu", "chl_graph.cu", "chl_tree.cu", "chl_small.cu", "chl_labels.cu", "chl_query.cu",
             "chl_serve.cu"]
+_HEADERS = ["chl_common.cuh", "chl_tree.cuh"]
 LIB_PATH = os.path.join(_HERE, "libchl.so")
 ARCH_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -65,7 +66,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
-    deps = _sources() + [os.path.join(_CSRC, "chl_common.cuh"), os.path.join(_INCLUDE, "chl.h")]
+    deps = _sources() + [os.path.join(_CSRC, h) for h in _HEADERS] + [os.path.join(_INCLUDE, "chl.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 

@@ -156,10 +156,12 @@ int Stage::n_idle = 0, Stage::made = 0;
 // updates sit on cache lines of their own
 struct Control {
     alignas(128) unsigned int next_root;
+    unsigned int next_spill;  // claim counter of the spilled roots (small_class)
     alignas(128) unsigned long long out_count;
     unsigned long long out_valid;
     alignas(128) unsigned int failed_count;
     unsigned int list_n;  // roots listed by the trivial-root split
+    unsigned int spill_n; // roots whose trees outgrew the shared-memory kernel
     int flags[2];
     unsigned long long stats[7];
 };
@@ -203,10 +205,25 @@ constexpr uint32_t DEFAULT_SMALL_TREE_EXPANSIONS = 8192;
 // scale 18 and 21: the phases after trees of 0.48 n and more gained, those
 // after trees of 0.43 n and less lost)
 constexpr double BIG_TREE_COVER = 0.45;
+// list memory of the tree slots above which a build takes fewer lists
+constexpr double STATE_BYTES = 24.0 * (1 << 30);
+// The shared-memory tree kernel runs a phase of at least SMALL_ROOTS roots whose
+// trees are expected to expand at most this many vertices on average (a phase of
+// fewer roots ends with the latency of its spilled trees: 5,400 roots of a
+// 128x128 grid took 0.50 instead of 0.38 ms). The largest class is for phases
+// without label pruning only: with it, the general kernel answers the queries of
+// a round with more warps (7,300 roots of R-MAT scale 16, 170 expansions each:
+// 0.51 ms there, 0.83 ms here).
+constexpr double SMALL_EXPANSIONS[SMALL_CLASSES] = {96, 300, 600};
+constexpr uint32_t SMALL_ROOTS = 16384;
 // shared memory per tree slot for the root's table distances by hub position in
 // the label-pruned phases: phases whose table holds at most 16,384 hubs look
 // each entry up with one load instead of a hash probe
 constexpr uint32_t ROOT_ARRAY_BYTES = 64u << 10;
+
+// vertices up to which a graph with short rows runs 128 instead of 256 threads
+// per tree
+constexpr uint32_t DIRECT_SMALL_N = 131072;
 
 struct Params {
     int tpt;
@@ -230,6 +247,7 @@ struct Params {
     uint32_t eta;  // Common Label Table hubs (0 = no table)
     uint32_t fin_words;  // settled-filter bitmap words per CTA
     uint32_t w_min;
+    int direct;  // short rows only (TreeLaunch::direct)
     uint32_t n;
     int max_slots() const { return std::max(slots, std::max(slots_lt, slots_sm)); }
     // list words per vertex over all slots, the largest of the launches' layouts
@@ -246,9 +264,19 @@ struct Params {
 // bucket rounds.
 Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_t free_bytes) {
     Params p;
-    p.tpt = o.threads_per_tree ? o.threads_per_tree : 1024;
+    p.direct = g.deg_max <= DIRECT_DEGREE;
+    // Threads per tree: trees of graphs with short rows expand about a hundred
+    // vertices a round, which 1024 threads leave mostly idle. Measured on grids
+    // (build ms at 64 / 128 / 256 / 1024 threads): 49,000 vertices 28.5 / 16.7 /
+    // 21.6 / 50.7, 262,000 vertices 406 / 190 / 172 / 375 (there more slots spill
+    // the last level cache).
+    p.tpt = o.threads_per_tree ? o.threads_per_tree : !p.direct ? 1024 : g.n <= DIRECT_SMALL_N ? 128 : 256;
     const double mean_deg = g.n ? double(g.m2) / double(g.n) : 0.0;
-    const double dflt = mean_deg >= 8.0 ? g.w_mean / 128.0 : 2.0 * g.w_mean;
+    // ... and where no weight lies far below the mean, buckets as wide as the
+    // lightest arc settle in one or two rounds instead of four (262,000-vertex
+    // grid at 256 threads: 193 ms at width 2048, 171 ms at 512, 231 ms at 256)
+    const double dflt = mean_deg >= 8.0 ? g.w_mean / 128.0
+                        : p.direct && g.w_min * 4.0 >= g.w_mean ? double(g.w_min) : 2.0 * g.w_mean;
     uint32_t d = 1;  // default: the power of two nearest to dflt
     while (double(d) * 1.5 < dflt && d < (1u << 30)) d <<= 1;
     if (o.bucket_delta > 0) d = uint32_t(o.bucket_delta);
@@ -281,6 +309,16 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     p.stage_want = o.query_stage_kb > 0 ? uint32_t(o.query_stage_kb) << 10 : 0u;
     plant_smem_split(p.tpt_lt, g.n, p.stage_want ? p.stage_want : ROOT_ARRAY_BYTES, &p.fin_words_lt,
                      &p.aux_lt);
+    // The lists are most of the slot state (n entries each). Past STATE_BYTES the
+    // build's memory outgrows what the pool keeps between builds, and each build
+    // maps gigabytes again (R-MAT scale 21: 55 GB, of which 36 GB for 608 slots
+    // of the small-tree launch; 75 of 800 ms), so large graphs take a narrower
+    // window, and the small-tree launch no more lists than the other launches.
+    {
+        const int per = plant_max_slots_per_sm(p.tpt, p.fin_words, 0);
+        const double slots1 = o.slots > 0 ? double(o.slots) : double(sms) * std::max(per, 1);
+        if (!o.window_buckets && slots1 * (4 + p.nwin) * 4.0 * double(g.n) > STATE_BYTES) p.nwin = 16;
+    }
     p.round_limit = o.round_limit ? o.round_limit : DEFAULT_ROUND_LIMIT;
     int per_sm = plant_max_slots_per_sm(p.tpt, p.fin_words, 0);
     if (per_sm < 1) per_sm = 1;
@@ -310,11 +348,26 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
         const long long cap_sm = (long long)(budget / per_slot_sm);
         if (o.slots <= 0 && slots_sm > cap_sm) slots_sm = cap_sm;
     }
+    if (o.slots <= 0 && double(slots_sm) * (4 + p.nwin_sm) * 4.0 * double(g.n) > STATE_BYTES) {
+        p.nwin_sm = std::min<uint32_t>(p.nwin_sm, 4);
+        const long long most = std::max(slots, slots_lt) * (4 + p.nwin) / (4 + p.nwin_sm);
+        if (slots_sm > most) slots_sm = most;
+    }
     if (slots_sm < 1) slots_sm = 1;
     p.slots_sm = int(slots_sm);
     p.slots = int(slots);
     p.slots_lt = int(slots_lt);
     return p;
+}
+
+// The class of the shared-memory tree kernel for a phase of `roots` roots whose
+// trees are expected to expand `est` vertices on average, or -1: the general
+// kernel
+int small_class(double est, uint64_t roots, bool label_pruned) {
+    if (roots < SMALL_ROOTS) return -1;
+    for (int c = 0; c < (label_pruned ? 2 : SMALL_CLASSES); ++c)
+        if (est <= SMALL_EXPANSIONS[c]) return c;
+    return -1;
 }
 
 struct DevBuf {
@@ -360,6 +413,7 @@ struct SlotState {
         tl.key = key.p;
         tl.key_bytes = P.kb;
         tl.w_min = P.w_min;
+        tl.direct = P.direct;
         tl.fin_words = P.fin_words;
         tl.fin_bits = P.fin_words * 32 < n ? P.fin_words * 32 : n;
         tl.rtag = (uint32_t *)tags.p;
@@ -593,7 +647,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     const uint64_t m2 = g->num_arcs;
     const uint64_t *d_row = g->row_ptr;
     const uint32_t *d_col = g->col, *d_w = g->w, *d_rank = rank;
-    DevBuf b_row, b_col, b_w, b_rank, b_ctl, b_ov, b_oh, b_od, b_op, b_fail, b_roots, b_ltroot;
+    DevBuf b_row, b_col, b_w, b_rank, b_ctl, b_ov, b_oh, b_od, b_op, b_fail, b_roots, b_ltroot, b_spill;
     const bool parents = (o.flags & CHL_FLAG_PARENTS) != 0;
     uint32_t *csr_parent = nullptr;
     SlotState slot;
@@ -617,6 +671,12 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     bool use_lt = false, hybrid = false, hybrid_off = false;
     bool small = false;  // later label-pruned phases run the small-tree launch
     bool big = false;    // the previous phase's trees were big (BIG_TREE_COVER)
+    // the next phase's class of the shared-memory tree kernel, from the sizes of
+    // the last phases' trees
+    int tiny = -1;
+    double exp_tree = 0.0;
+    const bool tiny_ok = o.mode == 0 && !o.small_threads_per_tree && o.query_stage_kb == 0 &&
+                         !(o.flags & CHL_FLAG_DENSE_ROOT_LABELS);
     uint64_t lt_phases = 0, small_phases = 0, overlapped = 0;
     uint64_t lt_records = 0;  // output records the label table holds
     const double psi_th = o.psi_threshold > 0.0f ? double(o.psi_threshold) : PSI_TH;
@@ -642,7 +702,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     for (auto &e : ev) CUDA_TRY(cudaEventCreate(&e));
     CUDA_TRY(cudaEventRecord(ev[0], s));
     b_row.s = b_col.s = b_w.s = b_rank.s = b_ctl.s = s;
-    b_ov.s = b_oh.s = b_od.s = b_op.s = b_fail.s = b_roots.s = b_ltroot.s = s;
+    b_ov.s = b_oh.s = b_od.s = b_op.s = b_fail.s = b_roots.s = b_ltroot.s = b_spill.s = s;
 
     // inputs on the device
     if (g->mem == CHL_MEM_HOST) {
@@ -746,6 +806,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     const uint64_t exp0 = agg[0], T0 = T, arc0 = agg[1], pr0 = agg[6], rd0 = agg[4], bk0 = agg[5];
     const uint64_t tr0 = agg[3], triv0 = agg[2];
     const bool ph_small = small;
+    const int ph_tiny = tiny;
     const bool ph_narrow = big && P.delta_big && lt.offsets;
     const int ph_lt = lt.offsets ? 1 : 0;
     if (trace) t_ph = now_ms();
@@ -828,7 +889,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
             // the filler's split listed this phase's roots and counts them on
             // the device; the filler's claim counter is shared
             CUDA_TRY(cudaStreamWaitEvent(s, fin.ev_split, 0));
-            if (small) CUDA_TRY(cudaStreamWaitEvent(s, fin.ev_done, 0));  // another slot layout
+            // another slot layout, or trees spilled to all slots
+            if (small || tiny >= 0) CUDA_TRY(cudaStreamWaitEvent(s, fin.ev_done, 0));
             Control *fctl = (Control *)fin.ctl.p;
             tl.root_list = (const uint32_t *)fin.roots.p;
             tl.root_begin = 0;
@@ -872,6 +934,20 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
                     CUDA_TRY(launch_plant_trees(one, P.tpt, 1, s));
                     ++launches;
                 }
+            } else if (first && tiny >= 0) {
+                // trees in shared memory, then the roots that did not fit
+                if (!b_spill.p) CUDA_TRY(dmalloc(&b_spill.p, size_t(re - rb + 1) * 4, s));
+                CUDA_TRY(launch_plant_small(tl, tiny, o.slots > 0 ? std::min(count, uint32_t(o.slots)) : count,
+                                            (uint32_t *)b_spill.p, &ctl->spill_n, s));
+                TreeLaunch ts = tl;
+                ts.root_list = (const uint32_t *)b_spill.p;
+                ts.root_begin = 0;
+                ts.count_dev = &ctl->spill_n;
+                ts.next_root = &ctl->next_spill;
+                CUDA_TRY(lt.offsets ? launch_plant_trees(ts, small ? P.tpt_sm : P.tpt_lt,
+                                                         small ? P.slots_sm : P.slots_lt, s)
+                                    : launch_plant_trees(ts, P.tpt, P.slots, s));
+                launches += 2;
             } else if (lt.offsets) {
                 // the next phase's first trees fill this launch's tail (see Filler)
                 const uint64_t nx = std::min<uint64_t>(
@@ -1034,6 +1110,13 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
                 }
             }
             pending = failed;
+            if (first && tiny >= 0 && hc.spill_n > hc.next_spill) {
+                // spilled roots that no launch claimed
+                const size_t k = hc.spill_n - hc.next_spill;
+                pending.resize(failed.size() + k);
+                CUDA_TRY(cudaMemcpy(pending.data() + failed.size(), (const uint32_t *)b_spill.p + hc.next_spill, k * 4,
+                                    cudaMemcpyDeviceToHost));
+            }
             for (uint32_t i = claimed_upto; i < count; ++i) pending.push_back(root_at(i));
             first = false;
             if (attempt > 40) {
@@ -1053,7 +1136,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     // many vertices per label (Psi = expansions / labels above psi_th), or once
     // the Common Label Table pruned a large share of their expansions; before
     // that, the per-vertex table query would cost more than it saves.
-    if (hybrid && !use_lt && T > T0) {
+    if (hybrid && !use_lt && !hybrid_off && T > T0) {
         const double psi = double(agg[0] - exp0) / double(T - T0);
         const double cut = agg[0] > exp0 ? double(agg[6] - pr0) / double(agg[0] - exp0) : 0.0;
         const double ratio = m2 ? double(T) / double(m2) : 0.0;
@@ -1061,7 +1144,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         if (psi > psi_th || (P.eta && cut >= CLT_PRUNE_TH && o.psi_threshold == 0.0f)) use_lt = true;
         else if (ph == 0 && o.psi_threshold == 0.0f && o.switch_ratio >= 0.0f && ratio < ratio_th)
             use_lt = true;
-        // far down the ranking and still cheap trees: the rest is one phase
+        // far down the ranking and still cheap trees: no switch any more, and the
+        // rest is one phase, unless its small trees have a kernel of their own
         else if (pe >= std::max<uint64_t>(uint64_t(P.slots) * 8, 8192) && psi < psi_th / 2)
             hybrid_off = true;
     }
@@ -1098,10 +1182,20 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     // next phase's overlapped first trees (launched during it) rely on.
     if (hybrid && pe < re) {
         const uint64_t step_min = uint64_t(P.slots) * 2;
-        const uint64_t nx = hybrid_off ? re
+        const uint64_t nx = hybrid_off && !tiny_ok ? re
                             : ph == 0 ? uint64_t(pe) + P.slots
-                                      : std::max<uint64_t>(uint64_t(pe) * (use_lt && !ph_small ? 2 : 4), pe + step_min);
+                                      : std::max<uint64_t>(uint64_t(pe) * (use_lt && !ph_small && ph_tiny < 0 ? 2 : 4), pe + step_min);
         phases.push_back({pe, uint32_t(std::min<uint64_t>(nx, re))});
+    }
+    // the next phase's kernel: its trees are expected to be this phase's mean,
+    // shrunk as that shrank from the last phase's
+    {
+        const uint64_t built = (agg[3] - tr0) - (agg[2] - triv0);
+        const double mean = built ? double(agg[0] - exp0) / double(built) : 0.0;
+        const double shrink = exp_tree > 0.0 ? std::min(1.0, std::max(0.1, mean / exp_tree)) : 1.0;
+        tiny = tiny_ok && built && ph + 1 < phases.size()
+                   ? small_class(mean * shrink, phases[ph + 1].second - phases[ph + 1].first, use_lt) : -1;
+        exp_tree = mean;
     }
     double t_tree = trace ? now_ms() - t_ph : 0;
     if (use_lt && ph + 1 < phases.size()) {
@@ -1127,9 +1221,9 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     if (trace) {
         CUDA_TRY(cudaStreamSynchronize(s));
         std::fprintf(stderr,
-                     "chl phase %zu roots [%u, %u) table %d%s%s trees %.3f ms assemble %.3f ms "
+                     "chl phase %zu roots [%u, %u) table %d%s%s class %d spilled %u trees %.3f ms assemble %.3f ms "
                      "expanded %llu arcs %llu labels %llu rounds %llu buckets %llu pruned %llu\n",
-                     ph, pb, pe, ph_lt, ph_small ? " small" : "", ph_narrow ? " narrow" : "", t_tree,
+                     ph, pb, pe, ph_lt, ph_small ? " small" : "", ph_narrow ? " narrow" : "", ph_tiny, hc.spill_n, t_tree,
                      now_ms() - t_ph - t_tree,
                      (unsigned long long)(agg[0] - exp0), (unsigned long long)(agg[1] - arc0),
                      (unsigned long long)(T - T0), (unsigned long long)(agg[4] - rd0),

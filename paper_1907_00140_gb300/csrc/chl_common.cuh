@@ -34,10 +34,12 @@ struct RankGraph {
     uint32_t *vert_at = nullptr; // [n] pos -> caller vertex id
     uint32_t *pos_of = nullptr;  // [n] caller vertex id -> pos
     uint32_t w_max = 0, w_min = 0;
+    uint32_t deg_max = 0;        // longest row
     double w_mean = 0.0;
 };
 
 // ------------------------------------------------------------------ tree kernel interface
+constexpr uint32_t DIRECT_DEGREE = 8;
 struct TreeLaunch {
     // graph (rank order)
     uint32_t n;
@@ -55,6 +57,7 @@ struct TreeLaunch {
     int delta_shift;    // log2(delta) when delta is a power of two, else -1
     uint32_t nwin;
     uint32_t w_min;     // lightest arc weight
+    int direct;         // every row holds at most DIRECT_DEGREE arcs: a thread relaxes a whole row
     uint32_t round_limit;  // expansion rounds per tree before ERR_ROUND_LIMIT
     uint32_t fin_words; // settled-filter bitmap words in dynamic shared memory
     uint32_t fin_bits;  // vertices (pos) the bitmap covers: min(n, 32 * fin_words)
@@ -108,6 +111,15 @@ enum : int { ERR_NONE = 0, ERR_DIST_OVERFLOW = 1, ERR_ROUND_LIMIT = 2, ERR_WAIT_
 // launches (defined in chl_tree.cu)
 cudaError_t launch_plant_trees(const TreeLaunch &p, int threads_per_tree, int slots,
                                cudaStream_t s);
+// trees whose state fits shared memory (chl_small.cu): the same roots, pruning
+// and output, no slot state; roots whose trees outgrow class cls are appended to spill (*spill_n of them)
+constexpr int SMALL_CLASSES = 3;
+constexpr int SMALL_THREADS[SMALL_CLASSES] = {64, 64, 128};
+constexpr int SMALL_SLOTS[SMALL_CLASSES] = {512, 1024, 2048};
+// vertices a tree of the class may reach
+constexpr uint32_t small_capacity(int slots) { return uint32_t(slots) / 4 * 3; }
+cudaError_t launch_plant_small(const TreeLaunch &p, int cls, uint32_t max_trees, uint32_t *spill,
+                               unsigned int *spill_n, cudaStream_t s);
 // CTAs per SM of a launch with that bitmap and auxiliary area
 int plant_max_slots_per_sm(int threads_per_tree, uint32_t fin_words, uint32_t aux_bytes);
 // roots [begin, begin + count): the label of every trivial root is written to

@@ -197,22 +197,27 @@ __global__ void rank_perm_kernel(uint32_t n, const uint32_t *rank, const uint32_
     }
 }
 
-// degrees in rank order, and weight statistics
+struct WStats {
+    uint32_t wmax, wmin;
+    unsigned long long wsum;
+    uint32_t dmax;
+};
+
+// degrees in rank order, and the largest
 __global__ void rank_degree_kernel(uint32_t n, const uint64_t *row, const uint32_t *vert_at,
-                                   uint64_t *deg) {
+                                   uint64_t *deg, WStats *ws) {
+    uint32_t dmax = 0;
     for (uint64_t p = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < n;
          p += uint64_t(gridDim.x) * blockDim.x) {
         const uint32_t v = vert_at[p];
         deg[p] = row[v + 1] - row[v];
+        dmax = max(dmax, uint32_t(deg[p]));
     }
+    dmax = __reduce_max_sync(0xffffffffu, dmax);
+    if ((threadIdx.x & 31) == 0) atomicMax(&ws->dmax, dmax);
 }
 
-struct WStats {
-    uint32_t wmax, wmin;
-    unsigned long long wsum;
-};
-
-// one warp per vertex: copy its row with neighbours renumbered
+// one warp per vertex: copy its row with neighbours renumbered, weight statistics
 __global__ void rank_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t *col,
                                  const uint32_t *w, const uint32_t *vert_at,
                                  const uint32_t *pos_of, const uint64_t *nrow, uint2 *arc,
@@ -271,7 +276,7 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     uint32_t *cnt = nullptr;
     uint64_t *deg = nullptr;
     WStats *ws = nullptr;
-    WStats hws{0, 0xFFFFFFFFu, 0};
+    WStats hws{0, 0xFFFFFFFFu, 0, 0};
     g = RankGraph{};
     g.n = n;
     g.m2 = m2;
@@ -325,7 +330,7 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(dmalloc(&g.arc, (m2 ? m2 : 1) * sizeof(uint2), s));
     CK(dmalloc(&ws, sizeof(WStats), s));
     CK(cudaMemcpyAsync(ws, &hws, sizeof(WStats), cudaMemcpyHostToDevice, s));
-    rank_degree_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, row, g.vert_at, deg);
+    rank_degree_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, row, g.vert_at, deg, ws);
     *launches += 1;
     CK(cudaMemsetAsync(deg + n, 0, sizeof(uint64_t), s));
     CK(exclusive_scan_u64(deg, g.row, uint64_t(n) + 1, s, launches));
@@ -337,6 +342,7 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(cudaStreamSynchronize(s));
     g.w_max = m2 ? hws.wmax : 1;
     g.w_min = m2 ? hws.wmin : 1;
+    g.deg_max = hws.dmax;
     g.w_mean = m2 ? double(hws.wsum) / double(m2) : 1.0;
 done:
     if (chk) cudaFreeAsync(chk, s);

@@ -49,74 +49,16 @@
 #include <cstdio>
 
 #include "chl_common.cuh"
+#include "chl_tree.cuh"
 
 namespace chl {
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t NWIN_MAX = 64;
-constexpr uint32_t NONE = 0xFFFFFFFFu;
-constexpr uint32_t CLT_MAX = 64;  // largest Common Label Table (hubs)
-constexpr uint32_t LTH_SLOTS = 1024;  // hash of the root's labels in the label table
-constexpr uint32_t LTH_MAX = 512;     // most root labels the hash holds
-constexpr int QSTEPS = 4;             // label-table query from global memory: loads in flight per lane
 constexpr uint32_t WAIT_LIMIT = 1u << 22;  // polls of a staging barrier before it counts as hung
 #ifndef SMEM_CAP_BYTES
 #define SMEM_CAP_BYTES (132u << 10)
 #endif
-
-// ------------------------------------------------------------------ keys
-// Vertices are numbered by rank position (pos 0 = most important), so in the
-// tree of root h a vertex outranks h iff its pos is below h. Algorithm 3 keeps
-// per vertex its distance and the highest-ranked vertex a[v] on its shortest
-// paths; the label decision only asks whether a[v] is h itself, and a[v] can
-// never rank below h (every path starts at h). So one bit carries it:
-//   key = dist << 1 | clean
-// clean = 1 iff no vertex before v on the best known paths outranks h. Under
-// unsigned min a shorter distance wins and, at equal distance, clean = 0
-// wins: a vertex is outranked as soon as one of its shortest paths is (the
-// equal-distance branch of Algorithm 3; Sec. 5.2's example, a[v5] = v1).
-// v is live (would get the label (h, d)) iff clean and v >= h, and the bit
-// it passes on to its out-neighbours is exactly its own liveness.
-// Three layouts (K below is one of these traits; K::T is the stored word):
-//   KeyN  uint32  dist << 1 | clean            when every tentative distance is
-//                                              provably below 2^31 - 1 (the host
-//                                              checks w_max * n)
-//   KeyW  uint64  dist << 1 | clean            otherwise
-//   KeyP  uint64  dist << 32 | clean << 31 | parent, for path recovery (the
-//                 SPT parent stored with each label, Sec. 5.4 (Extensions)):
-//                 among equal (dist, clean) the smallest parent id wins, so
-//                 the parent is the lowest-numbered tight predecessor, a
-//                 deterministic choice. A candidate carries its source
-//                 vertex in the parent field.
-// All ones is "unreached".
-// U: arcs a lane relaxes per step of the arc pass (its loads in flight); the
-// 8-byte layouts take two, so that a thread's probe state fits its registers
-// at 1024 threads per SM.
-struct KeyN { using T = uint32_t; static constexpr int S = 1; static constexpr int U = 4; };
-struct KeyW { using T = uint64_t; static constexpr int S = 1; static constexpr int U = 2; };
-struct KeyP { using T = uint64_t; static constexpr int S = 32; static constexpr int U = 2; };
-
-template <typename K>
-__device__ __forceinline__ typename K::T key_inf() { return ~typename K::T(0); }
-template <typename K>
-__device__ __forceinline__ typename K::T make_key(uint64_t dist, bool clean, uint32_t parent) {
-    using KS = typename K::T;
-    return (KS(dist) << K::S) | (KS(clean) << (K::S - 1)) | (K::S > 1 ? KS(parent) : KS(0));
-}
-template <typename K>
-__device__ __forceinline__ uint32_t key_dist(typename K::T k) { return uint32_t(k >> K::S); }
-template <typename K>
-__device__ __forceinline__ bool key_clean(typename K::T k) { return (k >> (K::S - 1)) & 1; }
-template <typename K>
-__device__ __forceinline__ uint32_t key_parent(typename K::T k) {
-    return K::S > 1 ? uint32_t(k & 0x7FFFFFFFu) : 0u;
-}
-// largest distance a key holds below key_inf
-template <typename K>
-__device__ __forceinline__ uint64_t key_dist_limit() {
-    return sizeof(typename K::T) == 4 ? 0x7FFFFFFEull : 0xFFFFFFFEull;
-}
 
 struct Shared {
     uint32_t root;
@@ -156,11 +98,6 @@ struct Shared {
     uint32_t n_trees, n_trivial;
 };
 
-// bucket of a distance: a shift when the width is a power of two
-__device__ __forceinline__ uint32_t bucket_of(const TreeLaunch &p, uint32_t d) {
-    return p.delta_shift >= 0 ? d >> p.delta_shift : d / p.delta;
-}
-
 // A slot's lists sit back to back, n entries each: l0, l1, far, touch, then
 // the nwin window lists; their addresses are formed where used (fewer
 // registers held across the tree than one pointer per list).
@@ -176,11 +113,6 @@ struct Slot {
     __device__ __forceinline__ uint32_t *touch() const { return lists + 3 * size_t(n); }
     __device__ __forceinline__ uint32_t *sub(uint32_t s) const { return lists + (4 + size_t(s)) * n; }
 };
-
-template <typename K>
-__device__ __forceinline__ bool is_live(typename K::T k, uint32_t v, uint32_t h) {
-    return key_clean<K>(k) && v >= h;
-}
 
 // warp-aggregated append to a list counted by a shared-memory counter
 __device__ __forceinline__ void warp_append(bool pred, uint32_t val, uint32_t *list,
@@ -219,7 +151,6 @@ struct Probe {
     bool live;  // still worth committing
 };
 
-__device__ __forceinline__ uint32_t atomic_min_key(uint32_t *a, uint32_t v) { return atomicMin(a, v); }
 // atomicMin under a predicate, as one predicated instruction (no branch
 // around it); returns `none` where the predicate is false
 __device__ __forceinline__ uint32_t atomic_min_key_if(bool on, uint32_t *a, uint32_t v, uint32_t none) {
@@ -239,9 +170,6 @@ __device__ __forceinline__ uint64_t atomic_min_key_if(bool on, uint64_t *a, uint
         : "l"(a), "l"(v), "r"(uint32_t(on))
         : "memory");
     return old;
-}
-__device__ __forceinline__ uint64_t atomic_min_key(uint64_t *a, uint64_t v) {
-    return atomicMin((unsigned long long *)a, (unsigned long long)v);
 }
 __device__ __forceinline__ void atomic_set_key(uint32_t *a, uint32_t v) { atomicExch(a, v); }
 __device__ __forceinline__ void atomic_set_key(uint64_t *a, uint64_t v) {
@@ -499,87 +427,6 @@ __device__ __forceinline__ uint32_t owner(const Frontier<TPB, K> &F, uint64_t j,
     return lo;
 }
 
-// Common Label Table pruning (Sec. 5.3): the distance query between the root
-// and v over the table hubs, min_c d(h, c) + d(c, v); the table row of v is
-// read as 16-byte vectors (rows are padded to a multiple of 4 hubs)
-__device__ __forceinline__ uint64_t clt_query(const TreeLaunch &p, const Shared &S, uint32_t v) {
-    const uint4 *row = reinterpret_cast<const uint4 *>(p.hc + size_t(v) * p.hc_stride);
-    uint64_t best = ~0ull;
-    for (uint32_t c4 = 0; c4 < p.hc_stride / 4; ++c4) {
-        const uint4 x = __ldg(&row[c4]);
-        const uint32_t b[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t a = S.hch[c4 * 4 + j];
-            if (a != 0xFFFFFFFFu && b[j] != 0xFFFFFFFFu && uint64_t(a) + b[j] < best) best = uint64_t(a) + b[j];
-        }
-    }
-    return best;
-}
-
-// Label table of earlier phases (hybrid pruning): every label of every hub of
-// rank position below p.lt_hubs, as CSR by vertex rank position (entries of a
-// vertex unordered). min over shared hubs c of d(h,c) + d(c,v) <= dv means a
-// vertex outranking h lies on a shortest h-v path, as for the Common Label
-// Table: the table is complete for a rank-closed set of hubs (Sec. 5.3). The
-// query must see every table label of h and of v: a vertex reached only past a
-// pruned one is left with a wrong distance and ancestor unless it is pruned
-// too, which the complete query guarantees (a partial one would not). The
-// root's table labels are hashed in shared memory, or, when more than the hash
-// holds, written into the slot's dense array p.lt_root by hub position.
-__device__ __forceinline__ uint32_t lth_slot(uint32_t hp) { return (hp * 2654435761u) >> 22; }
-
-// does table entry (c, dc) of v witness dv: d(h, c) + dc <= dv for a hub c of
-// the root (its distance from the hash, or from the slot's dense array rootd)
-__device__ __forceinline__ bool lt_hit(const Shared &S, const uint32_t *rootd, uint32_t c, uint32_t dc,
-                                       uint32_t dv) {
-    if (dc > dv) return false;  // also every filler entry (all ones)
-    if (rootd) {
-        // written by this CTA at tree start: a plain load
-        const uint32_t dhc = rootd[c];
-        return dhc != NONE && uint64_t(dhc) + dc <= dv;
-    }
-    for (uint32_t sx = lth_slot(c);; sx = (sx + 1) & (LTH_SLOTS - 1)) {
-        const uint32_t key = S.lth_key[sx];
-        if (key == 0) return false;  // the hash holds at most half its slots
-        if (key == c + 1) return uint64_t(S.lth_val[sx]) + dc <= dv;
-    }
-}
-
-// One warp answers the query of one vertex whose table labels are entries
-// [a, b) in global memory: each lane takes every 32nd of them (coalesced),
-// QSTEPS steps of 32 are loaded before any is looked up, and the warp stops
-// at the first step where some lane found a witness.
-__device__ __forceinline__ bool lt_prunes_warp(const TreeLaunch &p, const Shared &S,
-                                               const uint32_t *rootd, uint64_t a, uint64_t b,
-                                               uint32_t dv, int lane) {
-    for (uint64_t j0 = a; j0 < b; j0 += 32 * QSTEPS) {
-        uint2 x[QSTEPS];
-#pragma unroll
-        for (int u = 0; u < QSTEPS; ++u) {
-            const uint64_t j = j0 + uint64_t(u) * 32 + lane;
-            x[u] = j < b ? __ldg(&p.lt_e[j]) : make_uint2(0, NONE);
-        }
-        bool hit = false;
-        if (rootd) {
-            // the root's distances by hub position: one predicated load per
-            // entry (no divergent region); fillers and entries beyond dv
-            // read nothing
-#pragma unroll
-            for (int u = 0; u < QSTEPS; ++u) {
-                const bool near = x[u].y <= dv;
-                const uint32_t dhc = near ? rootd[x[u].x] : NONE;
-                hit |= dhc != NONE && uint64_t(dhc) + x[u].y <= dv;
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < QSTEPS; ++u) hit |= lt_hit(S, rootd, x[u].x, x[u].y, dv);
-        }
-        if (__any_sync(0xffffffffu, hit)) return true;
-    }
-    return false;
-}
-
 // The same query over len entries already staged in shared memory.
 __device__ __forceinline__ bool lt_prunes_staged(const Shared &S, const uint32_t *rootd, const uint2 *e,
                                                  uint32_t len, uint32_t dv, int lane) {
@@ -683,6 +530,36 @@ __device__ void lt_answer(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F, u
     }
 }
 
+// Arc pass of a graph whose rows are all short (p.direct: at most DIRECT_DEGREE
+// arcs): each thread relaxes the row of the entry it staged, K::U arcs at a
+// time, so a round needs no degree prefix, no staged rows and no row search.
+// These graphs (road-like) expand a hundred vertices a round, so a round is
+// bound by its chain of dependent loads and barriers, not by balance.
+template <int TPB, typename K>
+__device__ __forceinline__ void direct_pass(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F,
+                                            const Slot<K> &sl, uint32_t h, uint64_t rs, uint32_t deg,
+                                            uint32_t dv, bool lv, uint32_t vid) {
+    using KS = typename K::T;
+    const int lane = threadIdx.x & 31;
+    // the keys of a list that is counted on entry are all read before any
+    // commit; the query queue is read out before the next chunk refills it
+    if (S.fuse_live || S.lt_prune) __syncthreads();
+    const uint32_t most = __reduce_max_sync(FULL, deg), arcs = __reduce_add_sync(FULL, deg);
+    if (lane == 0 && arcs) atomicAdd(&S.n_arcs, (unsigned long long)arcs);
+    const KS kv = make_key<K>(dv, lv, vid);
+    uint32_t bn = 0;  // improvements in the warp's buffer
+    for (uint32_t e = 0; e < most; e += K::U) {
+        uint2 a[K::U];
+#pragma unroll
+        for (int k = 0; k < K::U; ++k) a[k] = e + k < deg ? __ldg(&p.arc[rs + e + k]) : make_uint2(0, 0);
+        Probe<K> pr[K::U];
+#pragma unroll
+        for (int k = 0; k < K::U; ++k) probe(p, S, sl, kv, a[k], e + k < deg, pr[k]);
+        bn = commit_step<TPB, K>(p, S, F, sl, h, pr, bn);
+    }
+    if (bn) commit_buffer<TPB, K>(p, S, F, sl, h, bn);
+}
+
 // Expand the current list once, in chunks of TPB entries. In the first round
 // of a bucket the list is the bucket's window list, whose stale entries (keys
 // since lowered into an earlier bucket) are skipped.
@@ -769,8 +646,6 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
             deg = 0;
             if (clean) atomic_min_key(&sl.key[vid], make_key<K>(dv, false, 0));
         }
-        const bool ok = deg != 0;
-        const unsigned okm = __ballot_sync(FULL, ok);
         {
             const unsigned em = __ballot_sync(FULL, ex), pm = __ballot_sync(FULL, cut);
             if (lane == 0 && em) atomicAdd(&S.n_exp, (unsigned long long)__popc(em));
@@ -782,6 +657,12 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
             const int c = __popc(__ballot_sync(FULL, lv));
             if (lane == 0 && c) atomicSub(&S.cnt, c);
         }
+        if (p.direct) {
+            direct_pass<TPB, K>(p, S, F, sl, h, rs, uint32_t(deg), dv, lv, vid);
+            continue;
+        }
+        const bool ok = deg != 0;
+        const unsigned okm = __ballot_sync(FULL, ok);
         uint64_t inc = deg;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -894,6 +775,7 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
         }
         __syncthreads();  // the next chunk rewrites the staging arrays
     }
+    if (p.direct) __syncthreads();  // every list and counter of the round is complete
 }
 
 __device__ __forceinline__ uint32_t warp_min(uint32_t x) {

@@ -1,0 +1,172 @@
+// Device code shared by the tree kernels (chl_tree.cu, chl_small.cu): tree keys,
+// and the pruning queries over the Common Label Table and the label table.
+#pragma once
+
+#include "chl_common.cuh"
+
+namespace chl {
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr uint32_t NONE = 0xFFFFFFFFu;
+constexpr uint32_t CLT_MAX = 64;  // largest Common Label Table (hubs)
+constexpr uint32_t LTH_SLOTS = 1024;  // hash of the root's labels in the label table
+constexpr uint32_t LTH_MAX = 512;     // most root labels the hash holds
+constexpr int QSTEPS = 4;             // label-table query from global memory: loads in flight per lane
+
+// ------------------------------------------------------------------ keys
+// Vertices are numbered by rank position (pos 0 = most important), so in the
+// tree of root h a vertex outranks h iff its pos is below h. Algorithm 3 keeps
+// per vertex its distance and the highest-ranked vertex a[v] on its shortest
+// paths; the label decision only asks whether a[v] is h itself, and a[v] can
+// never rank below h (every path starts at h). So one bit carries it:
+//   key = dist << 1 | clean
+// clean = 1 iff no vertex before v on the best known paths outranks h. Under
+// unsigned min a shorter distance wins and, at equal distance, clean = 0
+// wins: a vertex is outranked as soon as one of its shortest paths is (the
+// equal-distance branch of Algorithm 3; Sec. 5.2's example, a[v5] = v1).
+// v is live (would get the label (h, d)) iff clean and v >= h, and the bit
+// it passes on to its out-neighbours is exactly its own liveness.
+// Three layouts (K below is one of these traits; K::T is the stored word):
+//   KeyN  uint32  dist << 1 | clean            when every tentative distance is
+//                                              provably below 2^31 - 1 (the host
+//                                              checks w_max * n)
+//   KeyW  uint64  dist << 1 | clean            otherwise
+//   KeyP  uint64  dist << 32 | clean << 31 | parent, for path recovery (the
+//                 SPT parent stored with each label, Sec. 5.4 (Extensions)):
+//                 among equal (dist, clean) the smallest parent id wins, so
+//                 the parent is the lowest-numbered tight predecessor, a
+//                 deterministic choice. A candidate carries its source
+//                 vertex in the parent field.
+// All ones is "unreached".
+// U: arcs a lane relaxes per step of the arc pass (its loads in flight); the
+// 8-byte layouts take two, so that a thread's probe state fits its registers
+// at 1024 threads per SM.
+struct KeyN { using T = uint32_t; static constexpr int S = 1; static constexpr int U = 4; };
+struct KeyW { using T = uint64_t; static constexpr int S = 1; static constexpr int U = 2; };
+struct KeyP { using T = uint64_t; static constexpr int S = 32; static constexpr int U = 2; };
+
+template <typename K>
+__device__ __forceinline__ typename K::T key_inf() { return ~typename K::T(0); }
+template <typename K>
+__device__ __forceinline__ typename K::T make_key(uint64_t dist, bool clean, uint32_t parent) {
+    using KS = typename K::T;
+    return (KS(dist) << K::S) | (KS(clean) << (K::S - 1)) | (K::S > 1 ? KS(parent) : KS(0));
+}
+template <typename K>
+__device__ __forceinline__ uint32_t key_dist(typename K::T k) { return uint32_t(k >> K::S); }
+template <typename K>
+__device__ __forceinline__ bool key_clean(typename K::T k) { return (k >> (K::S - 1)) & 1; }
+template <typename K>
+__device__ __forceinline__ uint32_t key_parent(typename K::T k) {
+    return K::S > 1 ? uint32_t(k & 0x7FFFFFFFu) : 0u;
+}
+// largest distance a key holds below key_inf
+template <typename K>
+__device__ __forceinline__ uint64_t key_dist_limit() {
+    return sizeof(typename K::T) == 4 ? 0x7FFFFFFEull : 0xFFFFFFFEull;
+}
+
+// bucket of a distance: a shift when the width is a power of two
+__device__ __forceinline__ uint32_t bucket_of(const TreeLaunch &p, uint32_t d) {
+    return p.delta_shift >= 0 ? d >> p.delta_shift : d / p.delta;
+}
+
+template <typename K>
+__device__ __forceinline__ bool is_live(typename K::T k, uint32_t v, uint32_t h) {
+    return key_clean<K>(k) && v >= h;
+}
+
+__device__ __forceinline__ uint32_t atomic_min_key(uint32_t *a, uint32_t v) { return atomicMin(a, v); }
+__device__ __forceinline__ uint64_t atomic_min_key(uint64_t *a, uint64_t v) {
+    return atomicMin((unsigned long long *)a, (unsigned long long)v);
+}
+// In the queries below SH is a kernel's shared state: hch[] (the root's table
+// row), lth_key[] and lth_val[] (the root's table labels, hashed).
+
+// Common Label Table pruning (Sec. 5.3): the distance query between the root
+// and v over the table hubs, min_c d(h, c) + d(c, v); the table row of v is
+// read as 16-byte vectors (rows are padded to a multiple of 4 hubs)
+template <typename SH>
+__device__ __forceinline__ uint64_t clt_query(const TreeLaunch &p, const SH &S, uint32_t v) {
+    const uint4 *row = reinterpret_cast<const uint4 *>(p.hc + size_t(v) * p.hc_stride);
+    uint64_t best = ~0ull;
+    for (uint32_t c4 = 0; c4 < p.hc_stride / 4; ++c4) {
+        const uint4 x = __ldg(&row[c4]);
+        const uint32_t b[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t a = S.hch[c4 * 4 + j];
+            if (a != 0xFFFFFFFFu && b[j] != 0xFFFFFFFFu && uint64_t(a) + b[j] < best) best = uint64_t(a) + b[j];
+        }
+    }
+    return best;
+}
+
+// Label table of earlier phases (hybrid pruning): every label of every hub of
+// rank position below p.lt_hubs, as CSR by vertex rank position (entries of a
+// vertex unordered). min over shared hubs c of d(h,c) + d(c,v) <= dv means a
+// vertex outranking h lies on a shortest h-v path, as for the Common Label
+// Table: the table is complete for a rank-closed set of hubs (Sec. 5.3). The
+// query must see every table label of h and of v: a vertex reached only past a
+// pruned one is left with a wrong distance and ancestor unless it is pruned
+// too, which the complete query guarantees (a partial one would not). The
+// root's table labels are hashed in shared memory, or, when more than the hash
+// holds, written into the slot's dense array p.lt_root by hub position.
+__device__ __forceinline__ uint32_t lth_slot(uint32_t hp) { return (hp * 2654435761u) >> 22; }
+
+// does table entry (c, dc) of v witness dv: d(h, c) + dc <= dv for a hub c of
+// the root (its distance from the hash, or from the slot's dense array rootd)
+template <typename SH>
+__device__ __forceinline__ bool lt_hit(const SH &S, const uint32_t *rootd, uint32_t c, uint32_t dc,
+                                       uint32_t dv) {
+    if (dc > dv) return false;  // also every filler entry (all ones)
+    if (rootd) {
+        // written by this CTA at tree start: a plain load
+        const uint32_t dhc = rootd[c];
+        return dhc != NONE && uint64_t(dhc) + dc <= dv;
+    }
+    for (uint32_t sx = lth_slot(c);; sx = (sx + 1) & (LTH_SLOTS - 1)) {
+        const uint32_t key = S.lth_key[sx];
+        if (key == 0) return false;  // the hash holds at most half its slots
+        if (key == c + 1) return uint64_t(S.lth_val[sx]) + dc <= dv;
+    }
+}
+
+// One warp answers the query of one vertex whose table labels are entries
+// [a, b) in global memory: each lane takes every 32nd of them (coalesced),
+// QSTEPS steps of 32 are loaded before any is looked up, and the warp stops
+// at the first step where some lane found a witness.
+template <typename SH>
+__device__ __forceinline__ bool lt_prunes_warp(const TreeLaunch &p, const SH &S,
+                                               const uint32_t *rootd, uint64_t a, uint64_t b,
+                                               uint32_t dv, int lane) {
+    for (uint64_t j0 = a; j0 < b; j0 += 32 * QSTEPS) {
+        uint2 x[QSTEPS];
+#pragma unroll
+        for (int u = 0; u < QSTEPS; ++u) {
+            const uint64_t j = j0 + uint64_t(u) * 32 + lane;
+            x[u] = j < b ? __ldg(&p.lt_e[j]) : make_uint2(0, NONE);
+        }
+        bool hit = false;
+        if (rootd) {
+            // the root's distances by hub position: one predicated load per
+            // entry (no divergent region); fillers and entries beyond dv
+            // read nothing
+#pragma unroll
+            for (int u = 0; u < QSTEPS; ++u) {
+                const bool near = x[u].y <= dv;
+                const uint32_t dhc = near ? rootd[x[u].x] : NONE;
+                hit |= dhc != NONE && uint64_t(dhc) + x[u].y <= dv;
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < QSTEPS; ++u) hit |= lt_hit(S, rootd, x[u].x, x[u].y, dv);
+        }
+        if (__any_sync(0xffffffffu, hit)) return true;
+    }
+    return false;
+}
+
+}  // namespace
+}  // namespace chl

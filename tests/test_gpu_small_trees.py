@@ -1,0 +1,101 @@
+"""Trees built in shared memory (phases of many tiny trees) and rows relaxed by
+one thread (graphs of degree at most 8), against the oracle: every key layout,
+trees that outgrow the table (spilled to the general kernel), roots with more
+table labels than their hash holds, and a label buffer that fills up while
+spilled roots wait. Integers: comparisons are exact."""
+import re
+
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1907_00140_gb300 as chl  # noqa: E402
+from test_gpu_parity import DG, dev, assert_same  # noqa: E402
+from test_gpu_query_blocks import graph_of  # noqa: E402
+
+
+def line_and_triples(line, triples, seed):
+    """A path ranked from one end to the other, its vertices spread over all
+    rank positions (the tree of its j-th vertex reaches the line - j after it,
+    whose lists hold all j before it), and many paths of three vertices."""
+    rng = np.random.default_rng(seed)
+    n = line + 3 * triples
+    a = np.concatenate([np.arange(line - 1), line + np.arange(triples) * 3, line + np.arange(triples) * 3 + 1])
+    b = a + 1
+    pos = np.empty(n, np.int64)
+    at = np.linspace(0, n - 1, line).astype(np.int64)
+    pos[:line] = at
+    pos[line:] = rng.permutation(np.setdiff1d(np.arange(n), at))
+    return graph_of(n, a, b, rng.integers(1, 60, len(a))), (n - 1 - pos).astype(np.uint32)
+
+
+def case(name):
+    if name == "line":
+        return line_and_triples(1500, 14000, seed=4)
+    if name == "ba40k":
+        g = W.barabasi_albert(40000, 2, seed=9, wlo=1, whi=100)
+        return g, W.degree_rank(g)
+    if name == "rmat16":
+        g = W.rmat(16, 4, seed=16, wlo=1, whi=255)
+        return g, W.degree_rank(g)
+    g = W.grid(280, 15600, seed=24)
+    return g, W.spt_count_rank(g, 16, seed=24)
+
+
+CLASSES = {"line": {0}, "ba40k": {0, 1}, "rmat16": {0, 1}, "grid280": {0, 1, 2}}
+
+
+@pytest.fixture(scope="module", params=list(CLASSES))
+def built(request):
+    g, rank = case(request.param)
+    return request.param, g, rank, O.build_labels(g, rank, "plant", threads=8)
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(flags=chl.CHL_FLAG_WIDE_KEYS), dict(flags=chl.CHL_FLAG_PARENTS),
+                                  dict(label_capacity=50000), dict(slots=40)],
+                         ids=["default", "wide", "parents", "full buffer", "slots"])
+def test_small_trees_equal_oracle(built, opts, capfd, monkeypatch):
+    name, g, rank, ref = built
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    L = chl.build_labels(DG(g), dev(rank), **opts)
+    seen = [(int(c), int(s)) for c, s in re.findall(r"class (-?\d+) spilled (\d+)", capfd.readouterr().err)]
+    assert_same(ref, *L.to_numpy())
+    assert any(c in CLASSES[name] for c, _ in seen), seen  # the shared-memory kernel ran
+    if name == "line":
+        assert any(s > 100 for _, s in seen), seen
+    if opts.get("flags") == chl.CHL_FLAG_PARENTS and name == "line":
+        off, hub, _ = L.to_numpy()
+        par = L.parents()
+        for v in (1, 700, 1499):  # the parent on a line ranked from its start is the vertex before
+            a, b = int(off[v]), int(off[v + 1])
+            assert np.array_equal(par[a:b], np.where(hub[a:b] == v, v, v - 1))
+
+
+@pytest.mark.parametrize("tpt", [32, 64, 128, 256, 512, 1024])
+@pytest.mark.parametrize("flags", [0, chl.CHL_FLAG_WIDE_KEYS, chl.CHL_FLAG_PARENTS])
+def test_short_rows_every_block_size(tpt, flags):
+    """Degrees 1 to 8 and a row length of 8 exactly: every block size and key layout."""
+    rng = np.random.default_rng(5)
+    n, deg = 3000, np.zeros(3000, np.int64)
+    e = set()
+    for u, v in rng.integers(0, n, (20000, 2)).tolist():
+        if u != v and deg[u] < 8 and deg[v] < 8 and (min(u, v), max(u, v)) not in e:
+            e.add((min(u, v), max(u, v)))
+            deg[u] += 1
+            deg[v] += 1
+    a, b = np.array(sorted(e)).T
+    g = graph_of(n, a, b, rng.integers(1, 30, len(a)))
+    assert deg.max() == 8 and deg.min() < 8
+    rank = W.degree_rank(g)
+    ref = O.build_labels(g, rank, "plant", threads=8)
+    L = chl.build_labels(DG(g), dev(rank), threads_per_tree=tpt, flags=flags)
+    assert_same(ref, *L.to_numpy())
