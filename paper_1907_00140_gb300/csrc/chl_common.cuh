@@ -157,7 +157,7 @@ cudaError_t assemble_labels(uint32_t n, uint64_t T, const uint32_t *in_v, const 
 // offsets [n+1] by rank position (pos_of maps caller ids to positions), entries
 // {hub position, distance} interleaved, each vertex's entries in no particular
 // order. Records of hubs below min_hub are left out. The entry array has two
-// spare entries past the last (all ones), so a read widened to 16-byte
+// spare entries past the last (never looked at), so a read widened to 16-byte
 // boundaries stays inside it.
 struct LabelTable {
     uint64_t *offsets = nullptr;

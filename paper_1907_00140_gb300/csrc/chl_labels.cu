@@ -6,12 +6,12 @@
 //   1. count labels per vertex (atomic histogram)
 //   2. exclusive scan -> offsets
 //   3. scatter (hubpos << 32 | dist) into each vertex's segment
-//   4. sort every segment by hubpos (= descending R of the hub): one warp per
-//      segment up to 32 labels, one CTA per segment up to MAX_SEGMENT labels
-//      (bitonic networks in shared memory); a longer segment (one CTA each) is
+//   4. sort every segment by hubpos (= descending R of the hub) and write it to
+//      the hub (caller id), hubpos and dist arrays: one warp per segment up to
+//      1024 labels (bitonic networks in registers), one CTA per segment up to
+//      MAX_SEGMENT labels (in shared memory); a longer segment (one CTA each) is
 //      sorted in chunks in shared memory, then the sorted runs are merged
 //      pairwise in global memory
-//   5. split into hub (caller id), hubpos and dist arrays
 #include "chl_common.cuh"
 
 namespace chl {
@@ -95,19 +95,143 @@ __global__ void scatter_kernel(uint64_t T, const uint32_t *v, const uint32_t *h,
     }
 }
 
-// classify segments by length into four work lists; record the longest
-__global__ void classify_kernel(uint32_t n, const uint64_t *off, uint32_t *small_list,
-                                uint32_t *mid_list, uint32_t *big_list, uint32_t *long_list,
-                                uint32_t *counts, unsigned long long *max_len) {
-    for (uint64_t v = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; v < n;
-         v += uint64_t(gridDim.x) * blockDim.x) {
-        const uint64_t len = off[v + 1] - off[v];
-        if (len <= 1) continue;
-        atomicMax(max_len, (unsigned long long)len);
-        if (len <= 32) small_list[atomicAdd(&counts[0], 1u)] = uint32_t(v);
-        else if (len <= 1024) mid_list[atomicAdd(&counts[1], 1u)] = uint32_t(v);
-        else if (len <= MAX_SEGMENT) big_list[atomicAdd(&counts[2], 1u)] = uint32_t(v);
-        else long_list[atomicAdd(&counts[3], 1u)] = uint32_t(v);
+// Segments by length: warp classes of up to 32, 128, 256, 512 and 1024 labels,
+// then one CTA's shared memory, then longer ones
+constexpr int CLASSES = 7, BIG = 5, LONG = 6;
+struct SortLists {
+    uint32_t *list;    // CLASSES lists of n vertices
+    uint32_t *counts;  // CLASSES counters
+    uint32_t n;
+    __device__ __forceinline__ const uint32_t *of(int c) const { return list + size_t(c) * n; }
+};
+
+// work lists of the segments that hold labels; records the longest
+__global__ void classify_kernel(SortLists w, const uint64_t *off, unsigned long long *max_len) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long most = 0;
+    for (uint64_t v0 = uint64_t(blockIdx.x) * blockDim.x + (threadIdx.x - lane); v0 < w.n;
+         v0 += uint64_t(gridDim.x) * blockDim.x) {
+        const uint64_t v = v0 + lane;
+        const uint64_t len = v < w.n ? off[v + 1] - off[v] : 0;
+        most = len > most ? len : most;
+        const int c = len == 0 ? -1 : len <= 32 ? 0 : len <= 128 ? 1 : len <= 256 ? 2 : len <= 512 ? 3
+                      : len <= 1024 ? 4 : len <= MAX_SEGMENT ? BIG : LONG;
+        const unsigned m = __match_any_sync(0xffffffffu, c);
+        const int leader = __ffs(m) - 1;
+        uint32_t b = 0;
+        if (c >= 0 && lane == leader) b = atomicAdd(&w.counts[c], uint32_t(__popc(m)));
+        b = __shfl_sync(0xffffffffu, b, leader);
+        if (c >= 0) w.list[size_t(c) * w.n + b + __popc(m & ((1u << lane) - 1))] = uint32_t(v);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, most, o);
+        most = x > most ? x : most;
+    }
+    if (lane == 0 && most) atomicMax(max_len, most);
+}
+
+// the label arrays a sorted segment is written to
+struct SortOut {
+    const uint32_t *vert_at;
+    uint32_t *hub, *hubpos, *dist;
+    __device__ __forceinline__ void put(uint64_t i, uint64_t k) const {
+        const uint32_t hp = uint32_t(k >> 32);
+        hubpos[i] = hp;
+        dist[i] = uint32_t(k);
+        hub[i] = __ldg(&vert_at[hp]);
+    }
+};
+
+// One warp sorts a segment of at most 32 * E keys (hubpos, dist) in registers:
+// lane l holds elements l * E .. l * E + E - 1 of the bitonic network, so only
+// the strides of E and more cross lanes (15 of 45 stages at 512 keys). The
+// sorted elements pass through shared memory, padded by one per lane, so that
+// they are written coalesced. buf: 32 * (E + 1) words of 8 bytes.
+//
+// Bound by instruction issue (about 3,000 warp instructions per 512 keys); the
+// network in shared memory with one CTA per segment that it replaces ran 45
+// stages with a barrier each.
+template <int E>
+__device__ __forceinline__ void sort_warp(uint32_t v, const uint64_t *off, const uint64_t *tmp, const SortOut &out,
+                                          uint64_t *buf) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t a = off[v];
+    const uint32_t len = uint32_t(off[v + 1] - a);
+    uint32_t h[E], d[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const uint32_t i = uint32_t(j) * 32 + lane;  // any order: the keys are unsorted
+        const uint64_t k = i < len ? __ldg(&tmp[a + i]) : ~0ull;
+        h[j] = uint32_t(k >> 32);
+        d[j] = uint32_t(k);
+    }
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1) {
+#pragma unroll
+        for (int s = k >> 1; s > 0; s >>= 1) {
+            if (s < E) {
+#pragma unroll
+                for (int j = 0; j < E; ++j) {
+                    const int q = j ^ s;
+                    if (q < j) continue;
+                    const bool up = k < E ? (j & k) == 0 : (lane & (k / E)) == 0;
+                    const bool swap = (h[j] > h[q]) == up;  // (equal only among fillers)
+                    const uint32_t hj = swap ? h[q] : h[j], hq = swap ? h[j] : h[q];
+                    const uint32_t dj = swap ? d[q] : d[j], dq = swap ? d[j] : d[q];
+                    h[j] = hj;
+                    h[q] = hq;
+                    d[j] = dj;
+                    d[q] = dq;
+                }
+            } else {
+                const int m = s / E;
+                const bool low = ((lane & m) == 0) == ((lane & (k / E)) == 0);  // keeps the smaller
+#pragma unroll
+                for (int j = 0; j < E; ++j) {
+                    const uint32_t oh = __shfl_xor_sync(0xffffffffu, h[j], m);
+                    const uint32_t od = __shfl_xor_sync(0xffffffffu, d[j], m);
+                    if ((oh < h[j]) == low) {
+                        h[j] = oh;
+                        d[j] = od;
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < E; ++j) buf[lane * (E + 1) + j] = uint64_t(h[j]) << 32 | d[j];
+    __syncwarp();
+    for (uint32_t i = lane; i < len; i += 32) out.put(a + i, buf[i + i / E]);
+    __syncwarp();  // the next segment reuses the buffer
+}
+
+constexpr int SORT_TPB = 128;
+
+// segments of up to 256 labels (classes 0 to 2), the longest class first
+__global__ void __launch_bounds__(SORT_TPB) sort_short_kernel(SortLists w, const uint64_t *off, const uint64_t *tmp,
+                                                              SortOut out) {
+    __shared__ uint64_t buf[SORT_TPB / 32][32 * 9];
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5, me = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t c2 = w.counts[2], c1 = c2 + w.counts[1], c0 = c1 + w.counts[0];
+    uint64_t *b = buf[threadIdx.x >> 5];
+    for (uint32_t i = me; i < c0; i += warps) {
+        if (i < c2) sort_warp<8>(w.of(2)[i], off, tmp, out, b);
+        else if (i < c1) sort_warp<4>(w.of(1)[i - c2], off, tmp, out, b);
+        else sort_warp<1>(w.of(0)[i - c1], off, tmp, out, b);
+    }
+}
+
+// segments of 257 to 1024 labels (classes 3 and 4), the longest class first
+__global__ void __launch_bounds__(SORT_TPB) sort_mid_kernel(SortLists w, const uint64_t *off, const uint64_t *tmp,
+                                                            SortOut out) {
+    __shared__ uint64_t buf[SORT_TPB / 32][32 * 33];
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5, me = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t c4 = w.counts[4], c3 = c4 + w.counts[3];
+    uint64_t *b = buf[threadIdx.x >> 5];
+    for (uint32_t i = me; i < c3; i += warps) {
+        if (i < c4) sort_warp<32>(w.of(4)[i], off, tmp, out, b);
+        else sort_warp<16>(w.of(3)[i - c4], off, tmp, out, b);
     }
 }
 
@@ -115,11 +239,11 @@ __global__ void classify_kernel(uint32_t n, const uint64_t *off, uint32_t *small
 // are sorted in shared memory (bitonic), then runs of width w, 2w, 4w, ...
 // are merged pairwise between tmp and tmp2 (each thread writes an equal share
 // of a merged pair, starting where the merge path of its first output crosses
-// the two runs); the sorted segment ends in tmp. Keys (hubpos << 32 | dist)
+// the two runs); the sorted segment goes to the label arrays. Keys (hubpos << 32 | dist)
 // are distinct within a segment (one label per hub), so the order is unique.
 __global__ void __launch_bounds__(1024) sort_long_kernel(const uint32_t *list, const uint32_t *count,
                                                          const uint64_t *off, uint64_t *tmp,
-                                                         uint64_t *tmp2) {
+                                                         uint64_t *tmp2, SortOut out) {
     __shared__ uint64_t sm[LONG_CHUNK];
     const uint32_t tid = threadIdx.x, nt = blockDim.x;
     for (uint32_t sidx = blockIdx.x; sidx < *count; sidx += gridDim.x) {
@@ -173,40 +297,17 @@ __global__ void __launch_bounds__(1024) sort_long_kernel(const uint32_t *list, c
             src = dst;
             dst = t;
         }
-        if (src != tmp + a)
-            for (uint64_t i = tid; i < len; i += nt) tmp[a + i] = src[i];
+        for (uint64_t i = tid; i < len; i += nt) out.put(a + i, src[i]);
         __syncthreads();
     }
 }
 
-// one warp per segment of <= 32 keys: bitonic network in registers
-__global__ void sort_small_kernel(const uint32_t *list, const uint32_t *count, const uint64_t *off,
-                                  uint64_t *tmp) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < *count; w += warps) {
-        const uint32_t v = list[w];
-        const uint64_t a = off[v], len = off[v + 1] - a;
-        uint64_t x = lane < len ? tmp[a + lane] : ~0ull;
-#pragma unroll
-        for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                const uint64_t y = __shfl_xor_sync(0xffffffffu, x, j);
-                const bool up = ((lane & k) == 0);
-                const bool lower = ((lane & j) == 0);
-                // keep min in the lower lane of an ascending pair
-                x = (lower == up) ? min(x, y) : max(x, y);
-            }
-        }
-        if (lane < len) tmp[a + lane] = x;
-    }
-}
-
 // one CTA per segment: bitonic sort in shared memory (size rounded up to a power of two)
-template <int TPB>
-__global__ void sort_block_kernel(const uint32_t *list, const uint32_t *count, const uint64_t *off,
-                                  uint64_t *tmp) {
+constexpr int BLOCK_TPB = 1024;
+__global__ void __launch_bounds__(BLOCK_TPB) sort_block_kernel(const uint32_t *list, const uint32_t *count,
+                                                               const uint64_t *off, const uint64_t *tmp,
+                                                               SortOut out) {
+    constexpr int TPB = BLOCK_TPB;
     extern __shared__ uint64_t sm[];
     for (uint32_t s = blockIdx.x; s < *count; s += gridDim.x) {
         const uint32_t v = list[s];
@@ -232,20 +333,8 @@ __global__ void sort_block_kernel(const uint32_t *list, const uint32_t *count, c
                 __syncthreads();
             }
         }
-        for (uint32_t i = threadIdx.x; i < len; i += TPB) tmp[a + i] = sm[i];
+        for (uint32_t i = threadIdx.x; i < len; i += TPB) out.put(a + i, sm[i]);
         __syncthreads();
-    }
-}
-
-__global__ void split_kernel(uint64_t T, const uint64_t *tmp, const uint32_t *vert_at,
-                             uint32_t *hub, uint32_t *hubpos, uint32_t *dist) {
-    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < T;
-         i += uint64_t(gridDim.x) * blockDim.x) {
-        const uint64_t k = tmp[i];
-        const uint32_t hp = uint32_t(k >> 32);
-        hubpos[i] = hp;
-        dist[i] = uint32_t(k);
-        hub[i] = vert_at[hp];
     }
 }
 
@@ -283,11 +372,11 @@ cudaError_t assemble_labels(uint32_t n, uint64_t T, const uint32_t *in_v, const 
     CKE(dmalloc(&out.dist, Tb * sizeof(uint32_t), s));
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(dmalloc(&tmp, Tb * sizeof(uint64_t), s));
-    CKE(dmalloc(&lists, 4 * size_t(n) * sizeof(uint32_t), s));
-    CKE(dmalloc(&counts, 4 * sizeof(uint32_t), s));
+    CKE(dmalloc(&lists, CLASSES * size_t(n) * sizeof(uint32_t), s));
+    CKE(dmalloc(&counts, CLASSES * sizeof(uint32_t), s));
     CKE(dmalloc(&maxlen, sizeof(unsigned long long), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
-    CKE(cudaMemsetAsync(counts, 0, 4 * sizeof(uint32_t), s));
+    CKE(cudaMemsetAsync(counts, 0, CLASSES * sizeof(uint32_t), s));
     CKE(cudaMemsetAsync(maxlen, 0, sizeof(unsigned long long), s));
     count_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, cnt);
     *launches += 1;
@@ -295,34 +384,38 @@ cudaError_t assemble_labels(uint32_t n, uint64_t T, const uint32_t *in_v, const 
     CKE(exclusive_scan_u64(cnt, out.offsets, uint64_t(n) + 1, s, launches));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     scatter_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, in_d, out.offsets, cnt, tmp);
-    classify_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, out.offsets, lists, lists + n,
-                                                     lists + 2 * size_t(n), lists + 3 * size_t(n),
-                                                     counts, maxlen);
-    *launches += 2;
-    CKE(cudaGetLastError());
-    CKE(cudaMemcpyAsync(&hmax, maxlen, sizeof(hmax), cudaMemcpyDeviceToHost, s));
-    CKE(cudaStreamSynchronize(s));
-    sort_small_kernel<<<sms * 8, 256, 0, s>>>(lists, counts, out.offsets, tmp);
-    sort_block_kernel<256><<<sms * 8, 256, 1024 * sizeof(uint64_t), s>>>(lists + n, counts + 1,
-                                                                         out.offsets, tmp);
-    *launches += 2;
-    if (hmax > 1024) {
-        // the attribute belongs to the current device: set on every call
-        CKE(cudaFuncSetAttribute(sort_block_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(MAX_SEGMENT * sizeof(uint64_t))));
-        sort_block_kernel<1024><<<sms, 1024, MAX_SEGMENT * sizeof(uint64_t), s>>>(
-            lists + 2 * size_t(n), counts + 2, out.offsets, tmp);
+    {
+        const SortLists w{lists, counts, n};
+        const SortOut so{vert_at, out.hub, out.hubpos, out.dist};
+        classify_kernel<<<grid_for(n, 256), 256, 0, s>>>(w, out.offsets, maxlen);
+        *launches += 2;
+        CKE(cudaGetLastError());
+        sort_short_kernel<<<sms * 8, SORT_TPB, 0, s>>>(w, out.offsets, tmp, so);
         *launches += 1;
-    }
-    if (hmax > MAX_SEGMENT) {
-        CKE(dmalloc(&tmp2, Tb * sizeof(uint64_t), s));
-        sort_long_kernel<<<sms, 1024, 0, s>>>(lists + 3 * size_t(n), counts + 3, out.offsets, tmp, tmp2);
-        *launches += 1;
+        if (n > 256) {  // (a list holds at most n labels)
+            sort_mid_kernel<<<sms * 4, SORT_TPB, 0, s>>>(w, out.offsets, tmp, so);
+            *launches += 1;
+        }
+        CKE(cudaGetLastError());
+        if (n > 1024) {
+            CKE(cudaMemcpyAsync(&hmax, maxlen, sizeof(hmax), cudaMemcpyDeviceToHost, s));
+            CKE(cudaStreamSynchronize(s));
+        }
+        if (hmax > 1024) {
+            // the attribute belongs to the current device: set on every call
+            CKE(cudaFuncSetAttribute(sort_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     int(MAX_SEGMENT * sizeof(uint64_t))));
+            sort_block_kernel<<<sms, BLOCK_TPB, MAX_SEGMENT * sizeof(uint64_t), s>>>(
+                lists + BIG * size_t(n), counts + BIG, out.offsets, tmp, so);
+            *launches += 1;
+        }
+        if (hmax > MAX_SEGMENT) {
+            CKE(dmalloc(&tmp2, Tb * sizeof(uint64_t), s));
+            sort_long_kernel<<<sms, 1024, 0, s>>>(lists + LONG * size_t(n), counts + LONG, out.offsets, tmp, tmp2, so);
+            *launches += 1;
+        }
         CKE(cudaGetLastError());
     }
-    split_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, tmp, vert_at, out.hub, out.hubpos, out.dist);
-    *launches += 1;
-    CKE(cudaGetLastError());
 done:
     if (cnt) cudaFreeAsync(cnt, s);
     if (tmp) cudaFreeAsync(tmp, s);
@@ -350,7 +443,6 @@ cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const u
     out = LabelTable{};
     CKE(dmalloc(&out.offsets, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(dmalloc(&out.e, (size_t(T) + 2) * sizeof(uint2), s));
-    CKE(cudaMemsetAsync(out.e, 0xFF, (size_t(T) + 2) * sizeof(uint2), s));
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     count_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, pos_of, min_hub, cnt);
@@ -381,7 +473,6 @@ cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, cons
     const uint64_t dT = T - T0;
     CKE(dmalloc(&out.offsets, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(dmalloc(&out.e, (size_t(T) + 2) * sizeof(uint2), s));
-    CKE(cudaMemsetAsync(out.e, 0xFF, (size_t(T) + 2) * sizeof(uint2), s));
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     if (dT) {
