@@ -71,7 +71,7 @@ struct Tree {
     int ok;
     uint32_t n_out, n_put;
     unsigned long long base;
-    unsigned long long n_exp, n_arcs, n_pruned;
+    unsigned long long n_exp[TPB / 32], n_arcs[TPB / 32], n_pruned[TPB / 32];  // statistics per warp
     // label-pruned phases only (the launch leaves the rest out otherwise)
     uint32_t lth_key[LTH_SLOTS], lth_val[LTH_SLOTS];
     uint32_t lth_bit[ROOT_BITS / 32];  // by hub position modulo ROOT_BITS
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         S.id[i] = EMPTY;
         S.key[i] = key_inf<K>();
     }
-    if (tid == 0) S.n_exp = S.n_arcs = S.n_pruned = 0;
+    if (lane == 0) S.n_exp[tid >> 5] = S.n_arcs[tid >> 5] = S.n_pruned[tid >> 5] = 0;
     unsigned long long n_rounds = 0, n_buckets = 0, n_trees = 0;
 
     for (;;) {
@@ -328,9 +328,9 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                         const unsigned em = __ballot_sync(FULL, ex), pm = __ballot_sync(FULL, cut);
                         const uint32_t arcs = __reduce_add_sync(FULL, deg);
                         if (lane == 0) {
-                            if (em) atomicAdd(&S.n_exp, (unsigned long long)__popc(em));
-                            if (pm) atomicAdd(&S.n_pruned, (unsigned long long)__popc(pm));
-                            if (arcs) atomicAdd(&S.n_arcs, (unsigned long long)arcs);
+                            S.n_exp[tid >> 5] += __popc(em);
+                            S.n_pruned[tid >> 5] += __popc(pm);
+                            S.n_arcs[tid >> 5] += arcs;
                         }
                     }
                     __syncthreads();
@@ -429,11 +429,12 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
             }
         }
     }
-    __syncthreads();
+    if (lane == 0) {
+        if (S.n_exp[tid >> 5]) atomicAdd(&p.stats[0], S.n_exp[tid >> 5]);
+        if (S.n_arcs[tid >> 5]) atomicAdd(&p.stats[1], S.n_arcs[tid >> 5]);
+        if (S.n_pruned[tid >> 5]) atomicAdd(&p.stats[6], S.n_pruned[tid >> 5]);
+    }
     if (tid == 0) {
-        atomicAdd(&p.stats[0], S.n_exp);
-        atomicAdd(&p.stats[1], S.n_arcs);
-        if (S.n_pruned) atomicAdd(&p.stats[6], S.n_pruned);
         atomicAdd(&p.stats[3], n_trees);
         atomicAdd(&p.stats[4], n_rounds);
         atomicAdd(&p.stats[5], n_buckets);

@@ -93,7 +93,7 @@ struct Shared {
     uint32_t slot;         // the tree slot this CTA holds
     // launch statistics of this CTA, reported once at exit (kept here, not in
     // registers, which the arc pass needs)
-    unsigned long long n_exp, n_arcs, n_pruned, n_rounds, n_buckets;
+    unsigned long long n_rounds, n_buckets;
     uint64_t lt_a, lt_b;   // the root's entries in the label table
     uint32_t n_trees, n_trivial;
 };
@@ -270,6 +270,9 @@ struct Frontier {
     typename K::T kv[TPB];  // make_key(distance, liveness, vertex) of the row's vertex
     uint32_t wrows[TPB / 32];
     uint64_t wdeg[TPB / 32];
+    // launch statistics per warp: a 64-bit shared counter that all warps add
+    // to is a loop of compare-and-swaps they contend in
+    unsigned long long n_exp[TPB / 32], n_arcs[TPB / 32], n_pruned[TPB / 32];
     // per warp: improvements waiting to be classified (vertex, new key, old key)
     uint32_t iu[TPB / 32][32];
     typename K::T ic[TPB / 32][32];
@@ -545,7 +548,7 @@ __device__ __forceinline__ void direct_pass(const TreeLaunch &p, Shared &S, Fron
     // commit; the query queue is read out before the next chunk refills it
     if (S.fuse_live || S.lt_prune) __syncthreads();
     const uint32_t most = __reduce_max_sync(FULL, deg), arcs = __reduce_add_sync(FULL, deg);
-    if (lane == 0 && arcs) atomicAdd(&S.n_arcs, (unsigned long long)arcs);
+    if (lane == 0) F.n_arcs[threadIdx.x >> 5] += arcs;
     const KS kv = make_key<K>(dv, lv, vid);
     uint32_t bn = 0;  // improvements in the warp's buffer
     for (uint32_t e = 0; e < most; e += K::U) {
@@ -648,8 +651,10 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
         }
         {
             const unsigned em = __ballot_sync(FULL, ex), pm = __ballot_sync(FULL, cut);
-            if (lane == 0 && em) atomicAdd(&S.n_exp, (unsigned long long)__popc(em));
-            if (lane == 0 && pm) atomicAdd(&S.n_pruned, (unsigned long long)__popc(pm));
+            if (lane == 0) {
+                F.n_exp[warp] += __popc(em);
+                F.n_pruned[warp] += __popc(pm);
+            }
         }
         // the bucket's live entries stop counting as pending when it is entered;
         // for a list of one chunk this stage counts them (no commit has run yet)
@@ -707,7 +712,7 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
         const uint64_t lo = per * warp;
         const uint64_t hi = lo + per < total ? lo + per : total;
         if (lo < hi) {
-            if (lane == 0) atomicAdd(&S.n_arcs, (unsigned long long)(hi - lo));
+            if (lane == 0) F.n_arcs[warp] += hi - lo;
             uint32_t oa = owner(F, lo, 0, nrows);
             uint32_t bn = 0;  // improvements in the warp's buffer
             for (uint64_t i0 = lo; i0 < hi; i0 += STEP) {
@@ -891,9 +896,10 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
     if (threadIdx.x == 0) {
         S.rid = p.slot_ctr[S.slot * 4 + 0];
         mbar_init(&S.mbar, TPB);
-        S.n_exp = S.n_arcs = S.n_pruned = S.n_rounds = S.n_buckets = 0;
+        S.n_rounds = S.n_buckets = 0;
         S.n_trees = S.n_trivial = 0;
     }
+    if ((threadIdx.x & 31) == 0) F.n_exp[threadIdx.x >> 5] = F.n_arcs[threadIdx.x >> 5] = F.n_pruned[threadIdx.x >> 5] = 0;
 
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1162,11 +1168,14 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
         __syncthreads();
     }
 
-    // counters (every warp's shared-memory adds came before the last barrier)
+    // counters
+    if ((threadIdx.x & 31) == 0) {
+        const int w = threadIdx.x >> 5;
+        if (F.n_exp[w]) atomicAdd(&p.stats[0], F.n_exp[w]);
+        if (F.n_arcs[w]) atomicAdd(&p.stats[1], F.n_arcs[w]);
+        if (F.n_pruned[w]) atomicAdd(&p.stats[6], F.n_pruned[w]);
+    }
     if (threadIdx.x == 0) {
-        atomicAdd(&p.stats[0], S.n_exp);
-        atomicAdd(&p.stats[1], S.n_arcs);
-        if (S.n_pruned) atomicAdd(&p.stats[6], S.n_pruned);
         atomicAdd(&p.stats[2], (unsigned long long)S.n_trivial);
         atomicAdd(&p.stats[3], (unsigned long long)S.n_trees);
         atomicAdd(&p.stats[4], S.n_rounds);
