@@ -216,6 +216,18 @@ constexpr double STATE_BYTES = 24.0 * (1 << 30);
 // 0.51 ms there, 0.83 ms here).
 constexpr double SMALL_EXPANSIONS[SMALL_CLASSES] = {96, 300, 600};
 constexpr uint32_t SMALL_ROOTS = 16384;
+// ... of at least this many vertices (77,000: 10.46 ms with it, 10.27 without;
+// 174,000: 41.0 and 41.4; 1.24 million: 698 and 767)
+constexpr uint32_t BIG_TREE_N = 131072;
+// graphs below this many vertices run their phases one after the other: the
+// second stream's launches cost more than the tails they fill (24,000 vertices:
+// 5.42 ms with them, 5.09 without; 50,000: 10.0 and 10.7)
+constexpr uint32_t OVERLAP_N = 32768;
+// hubs of the Common Label Table in the label-pruned phases of a build that asks
+// for the default size: every hub left out of the dense table is in the label
+// table, so the two prune alike, and a row per expanded vertex gets shorter
+// (R-MAT scale 18, 16 and 4 hubs: 41.0 and 39.6 ms; scale 21: 698 and 683)
+constexpr uint32_t LT_COMMON_HUBS = 4;
 // shared memory per tree slot for the root's table distances by hub position in
 // the label-pruned phases: phases whose table holds at most 16,384 hubs look
 // each entry up with one load instead of a hash probe
@@ -270,12 +282,25 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     // (build ms at 64 / 128 / 256 / 1024 threads): 49,000 vertices 28.5 / 16.7 /
     // 21.6 / 50.7, 262,000 vertices 406 / 190 / 172 / 375 (there more slots spill
     // the last level cache).
-    p.tpt = o.threads_per_tree ? o.threads_per_tree : !p.direct ? 1024 : g.n <= DIRECT_SMALL_N ? 128 : 256;
+    // Small graphs leave most of 1024 threads idle too (at 256 / 512 / 1024: 11,900
+    // arcs 0.95 / 1.04 / 1.06, 120,000 arcs 2.78 / 2.54 / 2.81, 190,000 arcs 2.43 /
+    // 1.99 / 1.74).
+    p.tpt = o.threads_per_tree ? o.threads_per_tree
+            : p.direct         ? (g.n <= DIRECT_SMALL_N ? 128 : 256)
+            : g.m2 <= 16384    ? 256
+            : g.m2 <= 131072   ? 512
+                               : 1024;
     const double mean_deg = g.n ? double(g.m2) / double(g.n) : 0.0;
     // ... and where no weight lies far below the mean, buckets as wide as the
     // lightest arc settle in one or two rounds instead of four (262,000-vertex
     // grid at 256 threads: 193 ms at width 2048, 171 ms at 512, 231 ms at 256)
-    const double dflt = mean_deg >= 8.0 ? g.w_mean / 128.0
+    // Scale-free: a round costs the latency of its loads and barriers, so a bucket
+    // should hold several hundred vertices; trees span about three mean weights
+    // (build ms by width: R-MAT scale 13, 2.50 at 1 and 1.68 at 32; scale 16, 7.8 at
+    // 1, 7.25 at 4 and 8, 8.0 at 16, and with weights to 100,000, 7.9 at 512, 7.7 at
+    // 1024, 8.5 at 2048; scale 17 with weights to 1000, 18.4 at 1, 14.1 at 8, 16.2
+    // at 32; scale 18, 41.0 at 1, 40.3 at 2; scale 21, 690 at 4 and at 8).
+    const double dflt = mean_deg >= 8.0 ? std::max(g.w_mean / 64.0, 1400.0 * g.w_mean / double(g.n))
                         : p.direct && g.w_min * 4.0 >= g.w_mean ? double(g.w_min) : 2.0 * g.w_mean;
     uint32_t d = 1;  // default: the power of two nearest to dflt
     while (double(d) * 1.5 < dflt && d < (1u << 30)) d <<= 1;
@@ -286,6 +311,7 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     p.delta_lt = o.pruned_bucket_delta > 0 ? uint32_t(o.pruned_bucket_delta) : dl;
     p.delta_big = o.big_tree_bucket_delta > 0   ? uint32_t(o.big_tree_bucket_delta)
                   : o.big_tree_bucket_delta < 0 ? 0u
+                        : g.n < BIG_TREE_N      ? 0u
                                                 : std::max<uint32_t>(1u, p.delta_lt / 16);
     p.nwin = o.window_buckets > 0 ? uint32_t(o.window_buckets) : 32;
     // 4-byte keys hold distances up to 2^31 - 2; every tentative distance of a
@@ -560,15 +586,15 @@ done:
 }
 
 // the same table from the records of a build whose first trees were the
-// table's roots (every label of hubs below eta is among the count records)
-chl_status table_from_records(const RankGraph &rg, const Params &P, const uint32_t *ov,
-                              const uint32_t *oh, const uint32_t *od, uint64_t count,
+// table's roots (every label of the first `hubs` hubs is among the count records)
+chl_status table_from_records(const RankGraph &rg, const uint32_t *ov,
+                              const uint32_t *oh, const uint32_t *od, uint64_t count, uint32_t hubs,
                               cudaStream_t s, CommonTable &t, int *launches) {
     chl_status st = CHL_OK;
     const uint32_t n = rg.n;
     t.buf.s = s;
-    t.hubs = P.eta;
-    t.stride = (P.eta + 3) & ~3u;
+    t.hubs = hubs;
+    t.stride = (hubs + 3) & ~3u;
     CUDA_TRY(dmalloc(&t.buf.p, size_t(n) * t.stride * 4, s));
     CUDA_TRY(cudaMemsetAsync(t.buf.p, 0xFF, size_t(n) * t.stride * 4, s));
     CUDA_TRY(launch_clt_fill(ov, oh, od, count, rg.pos_of, (uint32_t *)t.buf.p, t.stride, t.hubs, s));
@@ -788,7 +814,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     // earlier phases (a rank-closed hub set, so the labels stay canonical)
     // once the switch has fired. Other builds run as one phase.
     hybrid = rb == 0 && P.eta && !(o.flags & CHL_FLAG_NO_HYBRID) && re > P.eta;
-    overlap = hybrid && o.mode == 0 && o.overlap_phases >= 0;
+    overlap = hybrid && o.mode == 0 && o.overlap_phases >= 0 && n >= OVERLAP_N;
     // the Common Label Table is needed when some requested tree lies outside
     // it; a hybrid build takes it from its first phase instead
     if (P.eta && re > P.eta && !hybrid) {
@@ -1165,12 +1191,14 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         const uint64_t built = (agg[3] - tr0) - (agg[2] - triv0);
         big = built && double(agg[0] - exp0) / double(built) >= BIG_TREE_COVER * double(n);
     }
-    if (hybrid && !table.buf.p) {
+    const uint32_t table_hubs = use_lt && !o.common_hubs ? std::min(P.eta, LT_COMMON_HUBS) : P.eta;
+    if (hybrid && (!table.buf.p || (table.hubs != table_hubs && !lt.offsets))) {
         // the first phase built the table's trees: the Common Label Table from
-        // their labels, for every later phase
+        // their labels, for every later phase (a smaller one from the switch on)
+        table.buf.release();
         CUDA_TRY(cudaEventRecord(ev[5], s));
-        st = table_from_records(rg, P, (const uint32_t *)b_ov.p, (const uint32_t *)b_oh.p,
-                                (const uint32_t *)b_od.p, T, s, table, &launches);
+        st = table_from_records(rg, (const uint32_t *)b_ov.p, (const uint32_t *)b_oh.p,
+                                (const uint32_t *)b_od.p, T, table_hubs, s, table, &launches);
         if (st != CHL_OK) goto done;
         CUDA_TRY(cudaEventRecord(ev[6], s));
         with_table = true;

