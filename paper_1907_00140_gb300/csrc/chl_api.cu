@@ -163,7 +163,7 @@ struct Control {
     unsigned int list_n;  // roots listed by the trivial-root split
     unsigned int spill_n; // roots whose trees outgrew the shared-memory kernel
     int flags[2];
-    unsigned long long stats[7];
+    unsigned long long stats[8];
 };
 
 void bind_control(TreeLaunch &tl, Control *ctl) {
@@ -705,6 +705,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
                          !(o.flags & CHL_FLAG_DENSE_ROOT_LABELS);
     uint64_t lt_phases = 0, small_phases = 0, overlapped = 0;
     uint64_t lt_records = 0;  // output records the label table holds
+    unsigned long long max_dist = 0;  // largest label distance so far
     const double psi_th = o.psi_threshold > 0.0f ? double(o.psi_threshold) : PSI_TH;
     uint32_t claimed_upto = 0;
     bool first = true;
@@ -866,6 +867,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         if (lt.offsets) {
             tl.lt_off = lt.offsets;
             tl.lt_e = lt.e;
+            tl.lt_w = lt.w;
+            tl.lt_db = lt.db;
             tl.lt_hubs = pb;
             tl.lt_root = (uint32_t *)b_ltroot.p;
             tl.lt_hash_max = (o.flags & CHL_FLAG_DENSE_ROOT_LABELS) ? 0 : 0xFFFFFFFFu;
@@ -1047,6 +1050,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         CUDA_TRY(cudaMemcpyAsync(&hc, ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaStreamSynchronize(s));
         for (int k = 0; k < 7; ++k) agg[k] += hc.stats[k];
+        max_dist = std::max(max_dist, hc.stats[7]);
         if (hc.flags[0] == ERR_DIST_OVERFLOW) {
             st = set_error(CHL_EOVERFLOW, "a shortest distance reaches UINT32_MAX");
             goto done;
@@ -1068,6 +1072,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
             CUDA_TRY(cudaEventSynchronize(fin.ev_done));
             CUDA_TRY(cudaMemcpy(&fin.hc, fin.ctl.p, sizeof(Control), cudaMemcpyDeviceToHost));
             for (int k = 0; k < 7; ++k) agg[k] += fin.hc.stats[k];
+            max_dist = std::max(max_dist, fin.hc.stats[7]);
             overlapped += fin.hc.stats[3] - fin.hc.failed_count;
             if (fin.hc.flags[0] == ERR_DIST_OVERFLOW) {
                 st = set_error(CHL_EOVERFLOW, "a shortest distance reaches UINT32_MAX");
@@ -1239,13 +1244,15 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         // hubs of the Common Label Table are left out: every tree of a label-
         // pruned phase also queries that table, which holds all their labels
         const uint32_t min_hub = table.buf.p ? table.hubs : 0;
+        // (the staging copies take whole 8-byte entries)
+        const int db = P.stage_want ? 0 : table_dist_bits(pe, max_dist);
         if (!lt.offsets)
             CUDA_TRY(assemble_table(n, T, (const uint32_t *)b_ov.p, (const uint32_t *)b_oh.p,
-                                    (const uint32_t *)b_od.p, rg.pos_of, min_hub, lt, s, &launches));
+                                    (const uint32_t *)b_od.p, rg.pos_of, min_hub, db, lt, s, &launches));
         else
             CUDA_TRY(grow_table(n, lt, lt_records, T, (const uint32_t *)b_ov.p,
                                 (const uint32_t *)b_oh.p, (const uint32_t *)b_od.p, rg.pos_of, min_hub,
-                                s, &launches, fill[ph & 1].active ? &fill[ph & 1].old : nullptr));
+                                db, s, &launches, fill[ph & 1].active ? &fill[ph & 1].old : nullptr));
         lt_records = T;
     }
     if (trace) {

@@ -73,7 +73,9 @@ struct TreeLaunch {
     // rank position (offsets [n+1]) of {hub position, distance} entries, each
     // vertex's entries in no particular order (see LabelTable)
     const uint64_t *lt_off;
-    const uint2 *lt_e;     // {hub position, distance}
+    const uint2 *lt_e;     // {hub position, distance}, or
+    const uint32_t *lt_w;  // (lt_db > 0) hub position << lt_db | distance
+    int lt_db;
     uint32_t lt_hubs;
     uint32_t aux_bytes;    // dynamic shared memory after the settled bitmap (multiple of 128):
                            // the staging area, or the root's table distances by hub position
@@ -103,7 +105,8 @@ struct TreeLaunch {
     uint32_t *failed;          // roots whose labels did not fit
     unsigned int *failed_count;
     int *flags;                // [0] error code, [1] output full
-    unsigned long long *stats; // [0] expanded [1] arcs [2] trivial [3] trees [4] rounds [5] buckets [6] pruned
+    // [0] expanded [1] arcs [2] trivial [3] trees [4] rounds [5] buckets [6] pruned, [7] largest label distance
+    unsigned long long *stats;
 };
 
 enum : int { ERR_NONE = 0, ERR_DIST_OVERFLOW = 1, ERR_ROUND_LIMIT = 2, ERR_WAIT_LIMIT = 3 };
@@ -159,20 +162,32 @@ cudaError_t assemble_labels(uint32_t n, uint64_t T, const uint32_t *in_v, const 
 // order. Records of hubs below min_hub are left out. The entry array has two
 // spare entries past the last (never looked at), so a read widened to 16-byte
 // boundaries stays inside it.
+// Where every hub position and distance of the table fit 32 bits together, an
+// entry is one word (w; db bits of distance, below their all-ones value): the
+// queries read whole lists, and their time is the bytes of the lists.
 struct LabelTable {
     uint64_t *offsets = nullptr;
     uint2 *e = nullptr;
+    uint32_t *w = nullptr;
+    int db = 0;
 };
+// distance bits of packed entries for hub positions below hubs and distances up
+// to max_dist, or 0: they do not fit
+inline int table_dist_bits(uint32_t hubs, uint64_t max_dist) {
+    int hb = 1;
+    while (hb < 32 && (uint64_t(1) << hb) < hubs) ++hb;
+    return hb < 32 && max_dist < (uint64_t(1) << (32 - hb)) - 1 ? 32 - hb : 0;
+}
 cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const uint32_t *in_h,
                            const uint32_t *in_d, const uint32_t *pos_of, uint32_t min_hub,
-                           LabelTable &out, cudaStream_t s, int *launches);
+                           int db, LabelTable &out, cudaStream_t s, int *launches);
 
 // a table from assemble_table of records [0, T0) grown by records [T0, T):
 // each vertex keeps its old entries first (lt is replaced; on success the old
 // arrays are freed on s, or handed to *keep_old when that is non-null)
 cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, const uint32_t *in_v,
                        const uint32_t *in_h, const uint32_t *in_d, const uint32_t *pos_of,
-                       uint32_t min_hub, cudaStream_t s, int *launches, LabelTable *keep_old = nullptr);
+                       uint32_t min_hub, int db, cudaStream_t s, int *launches, LabelTable *keep_old = nullptr);
 void free_table(LabelTable &t, cudaStream_t s);
 
 // parents of label records into the slots of the assembled CSR (parent[T])

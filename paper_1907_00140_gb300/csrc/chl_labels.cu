@@ -40,15 +40,32 @@ __global__ void count_table_kernel(uint64_t T, const uint32_t *v, const uint32_t
         if (h[i] >= min_hub) atomicAdd((unsigned long long *)&cnt[pos_of[v[i]]], 1ull);
 }
 
+// the entries of a label table in either form
+struct TableEntries {
+    uint2 *e;
+    uint32_t *w;
+    int db;
+    explicit TableEntries(const LabelTable &t) : e(t.e), w(t.w), db(t.db) {}
+    __device__ __forceinline__ void put(uint64_t k, uint32_t hub, uint32_t dist) const {
+        if (db) w[k] = hub << db | dist;
+        else e[k] = make_uint2(hub, dist);
+    }
+    __device__ __forceinline__ uint2 get(uint64_t k) const {
+        if (!db) return e[k];
+        const uint32_t x = w[k];
+        return make_uint2(x >> db, x & ((1u << db) - 1));
+    }
+};
+
 __global__ void scatter_table_kernel(uint64_t T, const uint32_t *v, const uint32_t *h,
                                      const uint32_t *d, const uint32_t *pos_of, uint32_t min_hub,
-                                     const uint64_t *off, uint64_t *fill, uint2 *e) {
+                                     const uint64_t *off, uint64_t *fill, TableEntries e) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < T;
          i += uint64_t(gridDim.x) * blockDim.x) {
         if (h[i] < min_hub) continue;
         const uint32_t x = pos_of[v[i]];
         const uint64_t k = off[x] + atomicAdd((unsigned long long *)&fill[x], 1ull);
-        e[k] = make_uint2(h[i], d[i]);
+        e.put(k, h[i], d[i]);
     }
 }
 
@@ -60,13 +77,16 @@ __global__ void grown_count_kernel(uint32_t n, const uint64_t *old_off, uint64_t
 }
 
 // one warp per vertex: its old entries to the front of its new segment
-__global__ void copy_segments_kernel(uint32_t n, const uint64_t *old_off, const uint2 *old_e,
-                                     const uint64_t *new_off, uint2 *e) {
+__global__ void copy_segments_kernel(uint32_t n, const uint64_t *old_off, TableEntries old_e,
+                                     const uint64_t *new_off, TableEntries e) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
     for (uint64_t v = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
         const uint64_t a = old_off[v], len = old_off[v + 1] - a, o = new_off[v];
-        for (uint64_t i = lane; i < len; i += 32) e[o + i] = old_e[a + i];
+        for (uint64_t i = lane; i < len; i += 32) {
+            const uint2 x = old_e.get(a + i);
+            e.put(o + i, x.x, x.y);
+        }
     }
 }
 
@@ -74,14 +94,14 @@ __global__ void copy_segments_kernel(uint32_t n, const uint64_t *old_off, const 
 __global__ void scatter_new_kernel(uint64_t T0, uint64_t T, const uint32_t *v, const uint32_t *h,
                                    const uint32_t *d, const uint32_t *pos_of, uint32_t min_hub,
                                    const uint64_t *old_off, const uint64_t *off, uint64_t *fill,
-                                   uint2 *e) {
+                                   TableEntries e) {
     for (uint64_t i = T0 + uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < T;
          i += uint64_t(gridDim.x) * blockDim.x) {
         if (h[i] < min_hub) continue;
         const uint32_t x = pos_of[v[i]];
         const uint64_t k = off[x] + (old_off[x + 1] - old_off[x]) +
                            atomicAdd((unsigned long long *)&fill[x], 1ull);
-        e[k] = make_uint2(h[i], d[i]);
+        e.put(k, h[i], d[i]);
     }
 }
 
@@ -433,16 +453,21 @@ done:
     return e;
 }
 
+static cudaError_t alloc_entries(LabelTable &t, uint64_t T, int db, cudaStream_t s) {
+    t.db = db;
+    return db ? dmalloc(&t.w, (size_t(T) + 2) * sizeof(uint32_t), s) : dmalloc(&t.e, (size_t(T) + 2) * sizeof(uint2), s);
+}
+
 // Entries are allocated with two spare ones past the last, so that a read
 // widened to 16-byte boundaries (two entries) stays inside the array.
 cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const uint32_t *in_h,
                            const uint32_t *in_d, const uint32_t *pos_of, uint32_t min_hub,
-                           LabelTable &out, cudaStream_t s, int *launches) {
+                           int db, LabelTable &out, cudaStream_t s, int *launches) {
     cudaError_t e = cudaSuccess;
     uint64_t *cnt = nullptr;
     out = LabelTable{};
     CKE(dmalloc(&out.offsets, (size_t(n) + 1) * sizeof(uint64_t), s));
-    CKE(dmalloc(&out.e, (size_t(T) + 2) * sizeof(uint2), s));
+    CKE(alloc_entries(out, T, db, s));
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     count_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, pos_of, min_hub, cnt);
@@ -451,28 +476,26 @@ cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const u
     CKE(exclusive_scan_u64(cnt, out.offsets, uint64_t(n) + 1, s, launches));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     scatter_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, in_d, pos_of, min_hub,
-                                                          out.offsets, cnt, out.e);
+                                                          out.offsets, cnt, TableEntries(out));
     *launches += 1;
     CKE(cudaGetLastError());
 done:
     if (cnt) cudaFreeAsync(cnt, s);
     if (e != cudaSuccess) {
-        if (out.offsets) cudaFreeAsync(out.offsets, s);
-        if (out.e) cudaFreeAsync(out.e, s);
-        out = LabelTable{};
+        free_table(out, s);
     }
     return e;
 }
 
 cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, const uint32_t *in_v,
                        const uint32_t *in_h, const uint32_t *in_d, const uint32_t *pos_of,
-                       uint32_t min_hub, cudaStream_t s, int *launches, LabelTable *keep_old) {
+                       uint32_t min_hub, int db, cudaStream_t s, int *launches, LabelTable *keep_old) {
     cudaError_t e = cudaSuccess;
     uint64_t *cnt = nullptr;
     LabelTable out;
     const uint64_t dT = T - T0;
     CKE(dmalloc(&out.offsets, (size_t(n) + 1) * sizeof(uint64_t), s));
-    CKE(dmalloc(&out.e, (size_t(T) + 2) * sizeof(uint2), s));
+    CKE(alloc_entries(out, T, db, s));
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     if (dT) {
@@ -484,29 +507,27 @@ cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, cons
     *launches += 1;
     CKE(cudaGetLastError());
     CKE(exclusive_scan_u64(cnt, out.offsets, uint64_t(n) + 1, s, launches));
-    copy_segments_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, lt.offsets, lt.e,
-                                                                         out.offsets, out.e);
+    copy_segments_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, lt.offsets, TableEntries(lt),
+                                                                         out.offsets, TableEntries(out));
     *launches += 1;
     CKE(cudaGetLastError());
     if (dT) {
         CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
         scatter_new_kernel<<<grid_for(dT, 256), 256, 0, s>>>(T0, T, in_v, in_h, in_d, pos_of, min_hub,
-                                                             lt.offsets, out.offsets, cnt, out.e);
+                                                             lt.offsets, out.offsets, cnt, TableEntries(out));
         *launches += 1;
         CKE(cudaGetLastError());
     }
 done:
     if (cnt) cudaFreeAsync(cnt, s);
     if (e != cudaSuccess) {
-        if (out.offsets) cudaFreeAsync(out.offsets, s);
-        if (out.e) cudaFreeAsync(out.e, s);
+        free_table(out, s);
         return e;
     }
     if (keep_old) {
         *keep_old = lt;  // still read by trees on another stream: the caller frees it after them
     } else {
-        cudaFreeAsync(lt.offsets, s);
-        cudaFreeAsync(lt.e, s);
+        free_table(lt, s);
     }
     lt = out;
     return e;
@@ -515,6 +536,7 @@ done:
 void free_table(LabelTable &t, cudaStream_t s) {
     if (t.offsets) cudaFreeAsync(t.offsets, s);
     if (t.e) cudaFreeAsync(t.e, s);
+    if (t.w) cudaFreeAsync(t.w, s);
     t = LabelTable{};
 }
 

@@ -70,6 +70,7 @@ struct Tree {
     int stop;                 // error: give up
     int ok;
     uint32_t n_out, n_put;
+    uint32_t max_d;           // largest label distance (all trees)
     unsigned long long base;
     unsigned long long n_exp[TPB / 32], n_arcs[TPB / 32], n_pruned[TPB / 32];  // statistics per warp
     // label-pruned phases only (the launch leaves the rest out otherwise)
@@ -145,7 +146,7 @@ __device__ __forceinline__ void append16(bool on, uint32_t val, uint16_t *list, 
 
 // Answers the chunk's m table queries, eight lanes each: every lane takes every
 // eighth entry of the list, eight loads in flight, and the group stops after a
-// step with a witness (see lt_prunes_warp, which a whole warp runs for one of
+// step with a witness (the general kernel's lt_scan runs a whole warp for one of
 // the longer lists of the larger trees).
 template <typename TR>
 __device__ __forceinline__ void answer_queries(const TreeLaunch &p, TR &S, uint32_t m) {
@@ -166,14 +167,14 @@ __device__ __forceinline__ void answer_queries(const TreeLaunch &p, TR &S, uint3
 #pragma unroll
             for (int t = 0; t < STEPS; ++t) {
                 const uint32_t j = j0 + t * LANES + l;
-                e[t] = !found && j < len ? __ldg(&p.lt_e[a + j]) : make_uint2(0, NONE);
+                e[t] = !found && j < len ? lt_entry(p, a + j) : make_uint2(0, NONE);
             }
             bool hit = false;
 #pragma unroll
             for (int t = 0; t < STEPS; ++t) {
                 // most entries are no hub of the root: one load tells
                 const bool on = e[t].y <= dv && (S.lth_bit[(e[t].x & (ROOT_BITS - 1)) >> 5] >> (e[t].x & 31) & 1u);
-                if (on) hit |= lt_hit(S, nullptr, e[t].x, e[t].y, dv);
+                if (on) hit |= lth_find(S, e[t].x) <= dv - e[t].y;  // (never for NONE: dv is below it)
             }
             const unsigned h = __ballot_sync(FULL, hit);
             found |= ((h >> (group * LANES)) & ((1u << LANES) - 1)) != 0;
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         S.id[i] = EMPTY;
         S.key[i] = key_inf<K>();
     }
+    if (tid == 0) S.max_d = 0;
     if (lane == 0) S.n_exp[tid >> 5] = S.n_arcs[tid >> 5] = S.n_pruned[tid >> 5] = 0;
     unsigned long long n_rounds = 0, n_buckets = 0, n_trees = 0;
 
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                 for (uint32_t i = tid; i < ROOT_BITS / 32; i += TPB) S.lth_bit[i] = 0;
                 __syncthreads();
                 for (uint32_t i = tid; i < cnt; i += TPB) {
-                    const uint2 e = __ldg(&p.lt_e[a + i]);
+                    const uint2 e = lt_entry(p, a + i);
                     atomicOr(&S.lth_bit[(e.x & (ROOT_BITS - 1)) >> 5], 1u << (e.x & 31));
                     for (uint32_t sx = lth_slot(e.x);; sx = (sx + 1) & (LTH_SLOTS - 1)) {
                         if (atomicCAS(&S.lth_key[sx], 0u, e.x + 1) == 0u) {
@@ -380,13 +382,20 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         ++n_trees;
         // ---- emission: count, reserve the tree's output range, write, reset
         const uint32_t nt = S.n_touch;
-        uint32_t mine = 0;
+        uint32_t mine = 0, far = 0;
         for (uint32_t i = tid; i < nt; i += TPB) {
             const uint32_t s = S.touch[i];
-            mine += is_live<K>(S.key[s], S.id[s] & ID_MASK, h);
+            const KS k = S.key[s];
+            const bool on = is_live<K>(k, S.id[s] & ID_MASK, h);
+            mine += on;
+            if (on) far = max(far, key_dist<K>(k));
         }
         mine = __reduce_add_sync(FULL, mine);
-        if (lane == 0 && mine) atomicAdd(&S.n_out, mine);
+        far = __reduce_max_sync(FULL, far);
+        if (lane == 0 && mine) {
+            atomicAdd(&S.n_out, mine);
+            atomicMax(&S.max_d, far);
+        }
         __syncthreads();
         if (tid == 0) {
             const uint32_t nlab = S.n_out;
@@ -438,6 +447,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         atomicAdd(&p.stats[3], n_trees);
         atomicAdd(&p.stats[4], n_rounds);
         atomicAdd(&p.stats[5], n_buckets);
+        atomicMax(&p.stats[7], (unsigned long long)S.max_d);
     }
 }
 

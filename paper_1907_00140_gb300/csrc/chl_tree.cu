@@ -96,6 +96,7 @@ struct Shared {
     unsigned long long n_rounds, n_buckets;
     uint64_t lt_a, lt_b;   // the root's entries in the label table
     uint32_t n_trees, n_trivial;
+    uint32_t max_d;        // largest label distance
 };
 
 // A slot's lists sit back to back, n entries each: l0, l1, far, touch, then
@@ -438,7 +439,7 @@ __device__ __forceinline__ bool lt_prunes_staged(const Shared &S, const uint32_t
         bool hit = false;
         if (j < len) {
             const uint2 x = e[j];
-            hit = lt_hit(S, rootd, x.x, x.y, dv);
+            hit = x.y <= dv && (rootd ? rootd[x.x] : lth_find(S, x.x)) <= dv - x.y;  // (never for NONE)
         }
         if (__any_sync(0xffffffffu, hit)) return true;
     }
@@ -455,6 +456,54 @@ __device__ __forceinline__ void stage_wait(const TreeLaunch &p, Shared &S, uint3
             S.abort = 1;
         }
         if (it >= 2 * WAIT_LIMIT) break;
+    }
+}
+
+// Answers those of the qn queued queries (see lt_answer) that were not staged: a
+// warp per query, in steps of 32 * QSTEPS entries: each lane takes every 32nd of
+// a step (coalesced), and the warp stops at the first step where some lane found
+// a witness. root(c) is the root's distance to hub position c, or NONE.
+//
+// Bound by the bytes of the lists: at 64 bytes per clock into an SM the 8-byte
+// entries of a list (78 on average in R-MAT scale 18's fourth phase) took 10 of
+// the 12 clocks that a query cost; more loads in flight, votes after every 32
+// entries and fewer instructions per look-up all measured within 1.5%. Hence
+// the packed form (PACKED: p.lt_w; a filler is all ones, above every entry).
+// With dc <= dv the sum of the two distances is compared as root(c) <= dv - dc,
+// which needs no wider arithmetic and which NONE never passes (dv is below it).
+template <bool PACKED, int TPB, typename K, typename F1>
+__device__ __forceinline__ void lt_scan(const TreeLaunch &p, Frontier<TPB, K> &F, uint32_t qn, F1 root) {
+    constexpr int NW = TPB / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int db = p.lt_db;
+    for (uint32_t q = warp; q < qn; q += NW) {
+        const uint64_t e = F.pre[q];
+        if (!(e >> 63)) continue;
+        uint64_t at = F.base[q] + lane;
+        int left = int(uint32_t(e >> 32) & 0x7FFFFFFFu) - lane;
+        const uint32_t dv = uint32_t(e);
+        bool found;
+        do {
+            uint2 x[QSTEPS];
+#pragma unroll
+            for (int u = 0; u < QSTEPS; ++u) {
+                if (PACKED) x[u].x = left > 32 * u ? __ldg(&p.lt_w[at + 32 * u]) : NONE;
+                else x[u] = left > 32 * u ? __ldg(&p.lt_e[at + 32 * u]) : make_uint2(0, NONE);
+            }
+            bool hit = false;
+#pragma unroll
+            for (int u = 0; u < QSTEPS; ++u) {
+                const uint32_t c = PACKED ? x[u].x >> db : x[u].x;
+                const uint32_t dc = PACKED ? x[u].x & ((1u << db) - 1) : x[u].y;
+                const bool near = dc <= dv && (!PACKED || x[u].x != NONE);  // false for every filler
+                const uint32_t dhc = near ? root(c) : NONE;
+                hit |= near && dhc <= dv - dc;
+            }
+            found = __any_sync(FULL, hit);
+            at += 32 * QSTEPS;
+            left -= 32 * QSTEPS;
+        } while (!found && left + lane > 0);
+        if (lane == 0) F.pre[q] = found;
     }
 }
 
@@ -522,15 +571,12 @@ __device__ void lt_answer(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F, u
         }
         __syncthreads();  // the next batch reuses the staging area
     }
-    for (uint32_t q = warp; q < qn; q += NW) {
-        const uint64_t e = F.pre[q];
-        if (!(e >> 63)) continue;
-        const uint64_t a = F.base[q];
-        const bool hit =
-            lt_prunes_warp(p, S, rootd, a, a + ((e >> 32) & 0x7FFFFFFFu), uint32_t(e), lane);
-        __syncwarp();
-        if (lane == 0) F.pre[q] = hit;
-    }
+    // (the slot's array was written by this CTA at tree start: plain loads)
+    auto any_root = [&](uint32_t c) { return rootd ? rootd[c] : lth_find(S, c); };
+    if (!p.lt_db) lt_scan<false>(p, F, qn, any_root);
+    else if (S.lt_dense == 2)
+        lt_scan<true>(p, F, qn, [&](uint32_t c) { return fin_bitmap[stage_offset(p.fin_words) / 4 + c]; });
+    else lt_scan<true>(p, F, qn, any_root);
 }
 
 // Arc pass of a graph whose rows are all short (p.direct: at most DIRECT_DEGREE
@@ -897,7 +943,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
         S.rid = p.slot_ctr[S.slot * 4 + 0];
         mbar_init(&S.mbar, TPB);
         S.n_rounds = S.n_buckets = 0;
-        S.n_trees = S.n_trivial = 0;
+        S.n_trees = S.n_trivial = S.max_d = 0;
     }
     if ((threadIdx.x & 31) == 0) F.n_exp[threadIdx.x >> 5] = F.n_arcs[threadIdx.x >> 5] = F.n_pruned[threadIdx.x >> 5] = 0;
 
@@ -967,13 +1013,13 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                 for (uint32_t c = threadIdx.x; c < p.lt_hubs; c += TPB) rs[c] = NONE;
                 __syncthreads();
                 for (uint64_t j = lt_a + threadIdx.x; j < lt_b; j += TPB) {
-                    const uint2 e = __ldg(&p.lt_e[j]);  // hub positions of the table lie below lt_hubs
+                    const uint2 e = lt_entry(p, j);  // hub positions of the table lie below lt_hubs
                     rs[e.x] = e.y;
                 }
             } else if (lt_dense) {
                 uint32_t *rootd = p.lt_root + so;
                 for (uint64_t j = lt_a + threadIdx.x; j < lt_b; j += TPB) {
-                    const uint2 e = __ldg(&p.lt_e[j]);
+                    const uint2 e = lt_entry(p, j);
                     rootd[e.x] = e.y;
                 }
             } else if (lt_prune) {
@@ -982,7 +1028,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                 const uint64_t a = lt_a;
                 const uint32_t cnt = uint32_t(lt_b - lt_a);
                 for (uint32_t i = threadIdx.x; i < cnt; i += TPB) {
-                    const uint2 e = __ldg(&p.lt_e[a + i]);
+                    const uint2 e = lt_entry(p, a + i);
                     for (uint32_t sx = lth_slot(e.x);; sx = (sx + 1) & (LTH_SLOTS - 1)) {
                         if (atomicCAS(&S.lth_key[sx], 0u, e.x + 1) == 0u) {
                             S.lth_val[sx] = e.y;
@@ -1096,7 +1142,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                 // reset and give up on this tree; the host reports the error
                 for (uint32_t i = threadIdx.x; i < S.touch_n; i += TPB) sl.key[sl.touch()[i]] = key_inf<K>();
                 if (S.lt_dense == 1)
-                    for (uint64_t j = S.lt_a + threadIdx.x; j < S.lt_b; j += TPB) p.lt_root[so + __ldg(&p.lt_e[j]).x] = NONE;
+                    for (uint64_t j = S.lt_a + threadIdx.x; j < S.lt_b; j += TPB) p.lt_root[so + lt_entry(p, j).x] = NONE;
                 __threadfence();
                 __syncthreads();
                 break;
@@ -1107,6 +1153,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
             }
             __syncthreads();
             const uint32_t nt = S.touch_n;
+            uint32_t far = 0;
             for (uint32_t base = 0; base < nt; base += TPB) {
                 const uint32_t i = base + threadIdx.x;
                 bool lv = false;
@@ -1117,6 +1164,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                     lv = is_live<K>(k, u, h);
                     d = key_dist<K>(k);
                     par = key_parent<K>(k);
+                    if (lv) far = max(far, d);
                 }
                 const unsigned m = __ballot_sync(FULL, lv);
                 if (m) {
@@ -1132,12 +1180,14 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                     }
                 }
             }
+            far = __reduce_max_sync(FULL, far);
+            if ((threadIdx.x & 31) == 0 && far) atomicMax(&S.max_d, far);
             __syncthreads();
             nlab = S.out_n;
             // reset exactly what this tree modified
             for (uint32_t i = threadIdx.x; i < nt; i += TPB) sl.key[sl.touch()[i]] = key_inf<K>();
             if (S.lt_dense == 1)
-                for (uint64_t j = S.lt_a + threadIdx.x; j < S.lt_b; j += TPB) p.lt_root[so + __ldg(&p.lt_e[j]).x] = NONE;
+                for (uint64_t j = S.lt_a + threadIdx.x; j < S.lt_b; j += TPB) p.lt_root[so + lt_entry(p, j).x] = NONE;
             // the next tree reads keys with L2 loads and L2 atomics: the plain
             // reset stores must be visible there first, not only inside the CTA
             __threadfence();
@@ -1180,6 +1230,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
         atomicAdd(&p.stats[3], (unsigned long long)S.n_trees);
         atomicAdd(&p.stats[4], S.n_rounds);
         atomicAdd(&p.stats[5], S.n_buckets);
+        atomicMax(&p.stats[7], (unsigned long long)S.max_d);
         p.slot_ctr[S.slot * 4 + 0] = S.rid;
         if (p.dyn_slots) {
             // the slot is idle again (every key and root array entry reset)
@@ -1288,7 +1339,7 @@ cudaError_t launch_plant_trees(const TreeLaunch &pl, int tpt, int slots, cudaStr
     p.nslots = uint32_t(slots);
     if (p.nwin < 2 || p.nwin > NWIN_MAX) return cudaErrorInvalidValue;
     // the staging copies read the label table in 16-byte units
-    if (p.lt_off && ((reinterpret_cast<uintptr_t>(p.lt_e) & 15) || (p.stage_bytes & 15)))
+    if (p.lt_off && p.stage_bytes && (p.lt_db || (reinterpret_cast<uintptr_t>(p.lt_e) & 15) || (p.stage_bytes & 15)))
         return cudaErrorMisalignedAddress;
     if (p.stage_bytes > p.aux_bytes) return cudaErrorInvalidValue;
     switch (tpt) {

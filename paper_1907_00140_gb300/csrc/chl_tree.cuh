@@ -115,57 +115,21 @@ __device__ __forceinline__ uint64_t clt_query(const TreeLaunch &p, const SH &S, 
 // holds, written into the slot's dense array p.lt_root by hub position.
 __device__ __forceinline__ uint32_t lth_slot(uint32_t hp) { return (hp * 2654435761u) >> 22; }
 
-// does table entry (c, dc) of v witness dv: d(h, c) + dc <= dv for a hub c of
-// the root (its distance from the hash, or from the slot's dense array rootd)
-template <typename SH>
-__device__ __forceinline__ bool lt_hit(const SH &S, const uint32_t *rootd, uint32_t c, uint32_t dc,
-                                       uint32_t dv) {
-    if (dc > dv) return false;  // also every filler entry (all ones)
-    if (rootd) {
-        // written by this CTA at tree start: a plain load
-        const uint32_t dhc = rootd[c];
-        return dhc != NONE && uint64_t(dhc) + dc <= dv;
-    }
-    for (uint32_t sx = lth_slot(c);; sx = (sx + 1) & (LTH_SLOTS - 1)) {
-        const uint32_t key = S.lth_key[sx];
-        if (key == 0) return false;  // the hash holds at most half its slots
-        if (key == c + 1) return uint64_t(S.lth_val[sx]) + dc <= dv;
-    }
+// entry j of the label table: {hub position, distance}
+__device__ __forceinline__ uint2 lt_entry(const TreeLaunch &p, uint64_t j) {
+    if (!p.lt_db) return __ldg(&p.lt_e[j]);
+    const uint32_t x = __ldg(&p.lt_w[j]);
+    return make_uint2(x >> p.lt_db, x & ((1u << p.lt_db) - 1));
 }
 
-// One warp answers the query of one vertex whose table labels are entries
-// [a, b) in global memory: each lane takes every 32nd of them (coalesced),
-// QSTEPS steps of 32 are loaded before any is looked up, and the warp stops
-// at the first step where some lane found a witness.
+// the root's distance to hub position c by the hash, or NONE
 template <typename SH>
-__device__ __forceinline__ bool lt_prunes_warp(const TreeLaunch &p, const SH &S,
-                                               const uint32_t *rootd, uint64_t a, uint64_t b,
-                                               uint32_t dv, int lane) {
-    for (uint64_t j0 = a; j0 < b; j0 += 32 * QSTEPS) {
-        uint2 x[QSTEPS];
-#pragma unroll
-        for (int u = 0; u < QSTEPS; ++u) {
-            const uint64_t j = j0 + uint64_t(u) * 32 + lane;
-            x[u] = j < b ? __ldg(&p.lt_e[j]) : make_uint2(0, NONE);
-        }
-        bool hit = false;
-        if (rootd) {
-            // the root's distances by hub position: one predicated load per
-            // entry (no divergent region); fillers and entries beyond dv
-            // read nothing
-#pragma unroll
-            for (int u = 0; u < QSTEPS; ++u) {
-                const bool near = x[u].y <= dv;
-                const uint32_t dhc = near ? rootd[x[u].x] : NONE;
-                hit |= dhc != NONE && uint64_t(dhc) + x[u].y <= dv;
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < QSTEPS; ++u) hit |= lt_hit(S, rootd, x[u].x, x[u].y, dv);
-        }
-        if (__any_sync(0xffffffffu, hit)) return true;
+__device__ __forceinline__ uint32_t lth_find(const SH &S, uint32_t c) {
+    for (uint32_t sx = lth_slot(c);; sx = (sx + 1) & (LTH_SLOTS - 1)) {
+        const uint32_t key = S.lth_key[sx];
+        if (key == 0) return NONE;  // the hash holds at most half its slots
+        if (key == c + 1) return S.lth_val[sx];
     }
-    return false;
 }
 
 }  // namespace
