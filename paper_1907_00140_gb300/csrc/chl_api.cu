@@ -481,6 +481,8 @@ constexpr double PSI_TH = 16.0;
 // above which they do: where the top 16 hubs already cut that much, the labels
 // of every earlier hub cut far more and the per-vertex query pays
 constexpr double CLT_PRUNE_TH = 0.10;
+// ... and below which the table is not worth its rows any more
+constexpr double CLT_KEEP = 0.01;
 // ... or, right after the first phase (one tree per slot), the labels it
 // produced per arc of the graph stay below this: scale-free graphs, whose top
 // hubs cover most shortest paths, give 1.4 to 3 and gain from pruning with
@@ -695,6 +697,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     std::vector<std::pair<uint32_t, uint32_t>> phases;
     LabelTable lt;  // labels of earlier phases (hybrid)
     bool use_lt = false, hybrid = false, hybrid_off = false;
+    bool table_off = false;  // the Common Label Table pruned next to nothing
     bool small = false;  // later label-pruned phases run the small-tree launch
     bool big = false;    // the previous phase's trees were big (BIG_TREE_COVER)
     // the next phase's class of the shared-memory tree kernel, from the sizes of
@@ -863,7 +866,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         tl.arc = rg.arc;
         tl.vert_at = rg.vert_at;
         slot.fill(P, n, tl);
-        table.fill(tl);
+        if (!table_off) table.fill(tl);
         if (lt.offsets) {
             tl.lt_off = lt.offsets;
             tl.lt_e = lt.e;
@@ -1182,6 +1185,13 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         else if (pe >= std::max<uint64_t>(uint64_t(P.slots) * 8, 8192) && psi < psi_th / 2)
             hybrid_off = true;
     }
+    // Before the switch the table costs a row per expanded vertex and saves what
+    // it prunes (grids: 0.5% of the expansions): below CLT_KEEP the later phases
+    // of a default build do without it.
+    if (hybrid && !use_lt && !o.common_hubs && table.buf.p && agg[0] > exp0)
+        table_off = double(agg[6] - pr0) < CLT_KEEP * double(agg[0] - exp0);
+    else if (use_lt)
+        table_off = false;
     // The small-tree switch: once a label-pruned phase's trees averaged fewer
     // than small_exp expansions (trees only shrink further down the ranking),
     // the later phases run more, smaller blocks per SM, which hides the

@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                             S.la[tid] = a;
                             S.dv[tid] = dv;
                         }
-                        cut = prune && clt_query(p, S, v) <= dv;
+                        cut = prune && clt_prunes(p, S, v, dv);
                         if (lt) {
                             cut |= v < p.lt_hubs;  // a table hub: the complete query would prune it
                             if (cut) len = 0;

@@ -652,7 +652,7 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
                 if (v < p.fin_bits && uint64_t(dv) < t_lo + p.w_min)
                     atomicOr(&fin_bitmap[v >> 5], 1u << (v & 31));
                 ex = true;
-                cut = S.prune && clt_query(p, S, v) <= dv;
+                cut = S.prune && clt_prunes(p, S, v, dv);
                 // a hub of the label table meets the root at the top vertex of
                 // their shortest paths, which outranks v and so is a table hub
                 // too: the complete query would find it

@@ -84,23 +84,22 @@ __device__ __forceinline__ uint64_t atomic_min_key(uint64_t *a, uint64_t v) {
 // In the queries below SH is a kernel's shared state: hch[] (the root's table
 // row), lth_key[] and lth_val[] (the root's table labels, hashed).
 
-// Common Label Table pruning (Sec. 5.3): the distance query between the root
-// and v over the table hubs, min_c d(h, c) + d(c, v); the table row of v is
-// read as 16-byte vectors (rows are padded to a multiple of 4 hubs)
+// Common Label Table pruning (Sec. 5.3): does the distance query between the
+// root and v over the table hubs, min_c d(h, c) + d(c, v), reach dv; the table
+// row of v is read as 16-byte vectors (rows are padded to a multiple of 4 hubs).
+// With d(c, v) <= dv the sum is compared without wider arithmetic, and a missing
+// label (all ones) on either side never passes: dv is below it.
 template <typename SH>
-__device__ __forceinline__ uint64_t clt_query(const TreeLaunch &p, const SH &S, uint32_t v) {
+__device__ __forceinline__ bool clt_prunes(const TreeLaunch &p, const SH &S, uint32_t v, uint32_t dv) {
     const uint4 *row = reinterpret_cast<const uint4 *>(p.hc + size_t(v) * p.hc_stride);
-    uint64_t best = ~0ull;
+    bool hit = false;
     for (uint32_t c4 = 0; c4 < p.hc_stride / 4; ++c4) {
         const uint4 x = __ldg(&row[c4]);
         const uint32_t b[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t a = S.hch[c4 * 4 + j];
-            if (a != 0xFFFFFFFFu && b[j] != 0xFFFFFFFFu && uint64_t(a) + b[j] < best) best = uint64_t(a) + b[j];
-        }
+        for (int j = 0; j < 4; ++j) hit |= (b[j] <= dv) & (S.hch[c4 * 4 + j] <= dv - b[j]);
     }
-    return best;
+    return hit;
 }
 
 // Label table of earlier phases (hybrid pruning): every label of every hub of
