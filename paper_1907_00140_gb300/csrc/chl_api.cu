@@ -555,6 +555,7 @@ chl_status build_common_table(const RankGraph &rg, const Params &P, const SlotSt
     tl.row = rg.row;
     tl.arc = rg.arc;
     tl.vert_at = rg.vert_at;
+    tl.pos = rg.vertex_pos();
     tl.root_list = nullptr;
     tl.root_begin = 0;
     tl.root_count = P.eta;
@@ -580,7 +581,7 @@ chl_status build_common_table(const RankGraph &rg, const Params &P, const SlotSt
     if (agg)
         for (int k = 0; k < 7; ++k) agg[k] += hc.stats[k];
     CUDA_TRY(launch_clt_fill((const uint32_t *)b_ov.p, (const uint32_t *)b_oh.p,
-                             (const uint32_t *)b_od.p, hc.out_count, rg.pos_of, (uint32_t *)t.buf.p,
+                             (const uint32_t *)b_od.p, hc.out_count, rg.index_of(), (uint32_t *)t.buf.p,
                              t.stride, t.hubs, s));
     ++*launches;
 done:
@@ -599,7 +600,7 @@ chl_status table_from_records(const RankGraph &rg, const uint32_t *ov,
     t.stride = (hubs + 3) & ~3u;
     CUDA_TRY(dmalloc(&t.buf.p, size_t(n) * t.stride * 4, s));
     CUDA_TRY(cudaMemsetAsync(t.buf.p, 0xFF, size_t(n) * t.stride * 4, s));
-    CUDA_TRY(launch_clt_fill(ov, oh, od, count, rg.pos_of, (uint32_t *)t.buf.p, t.stride, t.hubs, s));
+    CUDA_TRY(launch_clt_fill(ov, oh, od, count, rg.index_of(), (uint32_t *)t.buf.p, t.stride, t.hubs, s));
     ++*launches;
 done:
     return st;
@@ -710,6 +711,10 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     uint64_t lt_records = 0;  // output records the label table holds
     unsigned long long max_dist = 0;  // largest label distance so far
     const double psi_th = o.psi_threshold > 0.0f ? double(o.psi_threshold) : PSI_TH;
+    // block sizes given by the caller may have no kernel for its numbering
+    const bool keep_ids = o.mode == 0 && (!o.threads_per_tree || caller_ids_block(o.threads_per_tree)) &&
+                          (!o.pruned_threads_per_tree || caller_ids_block(o.pruned_threads_per_tree)) &&
+                          (!o.small_threads_per_tree || caller_ids_block(o.small_threads_per_tree));
     uint32_t claimed_upto = 0;
     bool first = true;
     Filler fill[2];                  // next-phase trees in a phase's tail, by phase parity
@@ -761,7 +766,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
             goto done;
         }
     }
-    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, rg, s, &launches);
+    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, keep_ids, rg, s, &launches);
     if (st != CHL_OK) goto done;
 
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
@@ -865,6 +870,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         tl.row = rg.row;
         tl.arc = rg.arc;
         tl.vert_at = rg.vert_at;
+        tl.pos = rg.vertex_pos();
         slot.fill(P, n, tl);
         if (!table_off) table.fill(tl);
         if (lt.offsets) {
@@ -1258,10 +1264,10 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         const int db = P.stage_want ? 0 : table_dist_bits(pe, max_dist);
         if (!lt.offsets)
             CUDA_TRY(assemble_table(n, T, (const uint32_t *)b_ov.p, (const uint32_t *)b_oh.p,
-                                    (const uint32_t *)b_od.p, rg.pos_of, min_hub, db, lt, s, &launches));
+                                    (const uint32_t *)b_od.p, rg.index_of(), min_hub, db, lt, s, &launches));
         else
             CUDA_TRY(grow_table(n, lt, lt_records, T, (const uint32_t *)b_ov.p,
-                                (const uint32_t *)b_oh.p, (const uint32_t *)b_od.p, rg.pos_of, min_hub,
+                                (const uint32_t *)b_oh.p, (const uint32_t *)b_od.p, rg.index_of(), min_hub,
                                 db, s, &launches, fill[ph & 1].active ? &fill[ph & 1].old : nullptr));
         lt_records = T;
     }
@@ -1739,6 +1745,7 @@ chl_status tree_trial(const RankGraph &rg, const Params &P, const CommonTable &t
     tl.row = rg.row;
     tl.arc = rg.arc;
     tl.vert_at = rg.vert_at;
+    tl.pos = rg.vertex_pos();
     tl.root_list = roots;
     tl.root_begin = 0;
     tl.root_count = count;
@@ -1824,7 +1831,7 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
         d_w = (const uint32_t *)b_w.p;
         d_rank = (const uint32_t *)b_rank.p;
     }
-    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, rg, s, &launches);
+    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, false, rg, s, &launches);
     if (st != CHL_OK) goto done;
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     {

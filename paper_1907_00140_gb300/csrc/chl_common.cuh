@@ -25,7 +25,9 @@ namespace chl {
 
 // ------------------------------------------------------------------ graph in rank order
 // The input graph renumbered by rank position: vertex p of this graph is the
-// vertex of rank position p (R = n-1-p) of the caller's graph.
+// vertex of rank position p (R = n-1-p) of the caller's graph. A graph whose
+// rows are short and whose numbering is local (see prepare_graph) keeps the
+// caller's numbering instead (caller_ids).
 struct RankGraph {
     uint32_t n = 0;
     uint64_t m2 = 0;             // arcs
@@ -35,17 +37,25 @@ struct RankGraph {
     uint32_t *pos_of = nullptr;  // [n] caller vertex id -> pos
     uint32_t w_max = 0, w_min = 0;
     uint32_t deg_max = 0;        // longest row
+    bool caller_ids = false;     // vertices numbered as by the caller
+    const uint32_t *vertex_pos() const { return caller_ids ? pos_of : nullptr; }
+    // index of a caller's vertex in this graph: null = as it is
+    const uint32_t *index_of() const { return caller_ids ? nullptr : pos_of; }
     double w_mean = 0.0;
 };
 
 // ------------------------------------------------------------------ tree kernel interface
 constexpr uint32_t DIRECT_DEGREE = 8;
+// block sizes whose kernels take a graph in the caller's numbering (the defaults
+// of the graphs that keep it)
+constexpr bool caller_ids_block(int threads) { return threads == 128 || threads == 256; }
 struct TreeLaunch {
     // graph (rank order)
     uint32_t n;
     const uint64_t *row;
     const uint2 *arc;
-    const uint32_t *vert_at;
+    const uint32_t *vert_at;    // [n] rank position -> caller vertex id
+    const uint32_t *pos;        // [n] vertex -> rank position, or null: vertices are rank positions
     // roots: pos ids root_list[i] (if non-null) or root_begin + i, i < root_count
     const uint32_t *root_list;
     uint32_t root_begin;
@@ -70,7 +80,7 @@ struct TreeLaunch {
     // label table of the earlier phases of a hybrid build, or lt_off = null:
     // all labels of the hubs of rank position in [hc_hubs, lt_hubs) (the
     // Common Label Table answers for the hubs below hc_hubs), CSR by vertex
-    // rank position (offsets [n+1]) of {hub position, distance} entries, each
+    // (offsets [n+1]) of {hub position, distance} entries, each
     // vertex's entries in no particular order (see LabelTable)
     const uint64_t *lt_off;
     const uint2 *lt_e;     // {hub position, distance}, or
@@ -140,7 +150,7 @@ void plant_smem_split(int threads_per_tree, uint32_t n, uint32_t aux_want, uint3
                       uint32_t *aux_bytes);
 // Common Label Table entries from label records (those of hub positions < hubs)
 cudaError_t launch_clt_fill(const uint32_t *out_v, const uint32_t *out_h, const uint32_t *out_d,
-                            unsigned long long count, const uint32_t *pos_of, uint32_t *hc,
+                            unsigned long long count, const uint32_t *index_of, uint32_t *hc,
                             uint32_t stride, uint32_t hubs, cudaStream_t s);
 
 // label assembly (chl_labels.cu)
@@ -157,7 +167,7 @@ cudaError_t assemble_labels(uint32_t n, uint64_t T, const uint32_t *in_v, const 
                             int *too_long, cudaStream_t s, int *launches);
 
 // The same records as a table for the distance queries of label pruning:
-// offsets [n+1] by rank position (pos_of maps caller ids to positions), entries
+// offsets [n+1] by vertex of the tree graph (index_of maps caller ids, null = as they are), entries
 // {hub position, distance} interleaved, each vertex's entries in no particular
 // order. Records of hubs below min_hub are left out. The entry array has two
 // spare entries past the last (never looked at), so a read widened to 16-byte
@@ -179,14 +189,14 @@ inline int table_dist_bits(uint32_t hubs, uint64_t max_dist) {
     return hb < 32 && max_dist < (uint64_t(1) << (32 - hb)) - 1 ? 32 - hb : 0;
 }
 cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const uint32_t *in_h,
-                           const uint32_t *in_d, const uint32_t *pos_of, uint32_t min_hub,
+                           const uint32_t *in_d, const uint32_t *index_of, uint32_t min_hub,
                            int db, LabelTable &out, cudaStream_t s, int *launches);
 
 // a table from assemble_table of records [0, T0) grown by records [T0, T):
 // each vertex keeps its old entries first (lt is replaced; on success the old
 // arrays are freed on s, or handed to *keep_old when that is non-null)
 cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, const uint32_t *in_v,
-                       const uint32_t *in_h, const uint32_t *in_d, const uint32_t *pos_of,
+                       const uint32_t *in_h, const uint32_t *in_d, const uint32_t *index_of,
                        uint32_t min_hub, int db, cudaStream_t s, int *launches, LabelTable *keep_old = nullptr);
 void free_table(LabelTable &t, cudaStream_t s);
 
@@ -253,8 +263,9 @@ cudaError_t exclusive_scan_u64(const uint64_t *in, uint64_t *out, uint64_t n, cu
 // graph preparation (chl_graph.cu)
 // validates the caller CSR (device copy) and rank; builds the rank-ordered graph
 // returns CHL_OK / CHL_EINVAL (with message) / CHL_ECUDA / CHL_ENOMEM
+// (keep_ids: the graph may stay in the caller's numbering)
 chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uint32_t *col,
-                         const uint32_t *w, const uint32_t *rank, RankGraph &g, cudaStream_t s,
+                         const uint32_t *w, const uint32_t *rank, bool keep_ids, RankGraph &g, cudaStream_t s,
                          int *launches);
 void free_graph(RankGraph &g, cudaStream_t s);
 

@@ -98,6 +98,8 @@ enum : uint32_t {
 struct Check {
     uint32_t bits;
     uint32_t where;  // a vertex where the first failure was seen (any)
+    uint32_t deg_max;  // longest row
+    unsigned long long gap; // sum of |u - v| over the arcs
     unsigned long long fp;  // symmetry fingerprint: sum of h(v, u, w) - h(u, v, w) over the arcs
 };
 
@@ -106,11 +108,15 @@ __device__ void fail(Check *c, uint32_t bit, uint32_t v) {
 }
 
 __global__ void check_rows_kernel(uint32_t n, uint64_t m2, const uint64_t *row, Check *c) {
+    uint64_t dmax = 0;
     for (uint64_t v = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; v < n;
          v += uint64_t(gridDim.x) * blockDim.x) {
         const uint64_t a = row[v], b = row[v + 1];
         if (a > b || b > m2 || (v == 0 && a != 0) || (v == n - 1 && b != m2)) fail(c, BAD_ROWPTR, uint32_t(v));
+        else dmax = max(dmax, b - a);
     }
+    const uint32_t d = __reduce_max_sync(0xffffffffu, uint32_t(min(dmax, uint64_t(0xFFFFFFFFu))));
+    if ((threadIdx.x & 31) == 0 && d) atomicMax(&c->deg_max, d);
 }
 
 // 64-bit mix of an arc (the splitmix64 finaliser of Steele, Lea and Flood)
@@ -133,7 +139,7 @@ __global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_
                                   const uint32_t *w, Check *c) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    unsigned long long fp = 0;
+    unsigned long long fp = 0, gap = 0;
     for (uint64_t v = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
         const uint64_t a = row[v], b = row[v + 1];
         for (uint64_t e = a + lane; e < b; e += 32) {
@@ -142,12 +148,17 @@ __global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_
             if (wt == 0) fail(c, BAD_WEIGHT, uint32_t(v));
             if (u == v) fail(c, BAD_SELF, uint32_t(v));
             if (e > a && col[e - 1] >= u) fail(c, BAD_ORDER, uint32_t(v));
+            gap += u > v ? u - v : v - u;
             fp += arc_hash(uint32_t(v), u, wt) - arc_hash(u, uint32_t(v), wt);
         }
     }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) fp += __shfl_xor_sync(0xffffffffu, fp, o);
+    for (int o = 16; o; o >>= 1) {
+        fp += __shfl_xor_sync(0xffffffffu, fp, o);
+        gap += __shfl_xor_sync(0xffffffffu, gap, o);
+    }
     if (lane == 0 && fp) atomicAdd(&c->fp, fp);
+    if (lane == 0 && gap) atomicAdd(&c->gap, gap);
 }
 
 // exact symmetry check, run only when the fingerprint is not 0: the reverse
@@ -200,24 +211,20 @@ __global__ void rank_perm_kernel(uint32_t n, const uint32_t *rank, const uint32_
 struct WStats {
     uint32_t wmax, wmin;
     unsigned long long wsum;
-    uint32_t dmax;
 };
 
-// degrees in rank order, and the largest
+// degrees in rank order
 __global__ void rank_degree_kernel(uint32_t n, const uint64_t *row, const uint32_t *vert_at,
-                                   uint64_t *deg, WStats *ws) {
-    uint32_t dmax = 0;
+                                   uint64_t *deg) {
     for (uint64_t p = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < n;
          p += uint64_t(gridDim.x) * blockDim.x) {
         const uint32_t v = vert_at[p];
         deg[p] = row[v + 1] - row[v];
-        dmax = max(dmax, uint32_t(deg[p]));
     }
-    dmax = __reduce_max_sync(0xffffffffu, dmax);
-    if ((threadIdx.x & 31) == 0) atomicMax(&ws->dmax, dmax);
 }
 
-// one warp per vertex: copy its row with neighbours renumbered, weight statistics
+// one warp per vertex: copy its row with neighbours renumbered (vert_at null: as
+// they are), weight statistics
 __global__ void rank_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t *col,
                                  const uint32_t *w, const uint32_t *vert_at,
                                  const uint32_t *pos_of, const uint64_t *nrow, uint2 *arc,
@@ -227,11 +234,11 @@ __global__ void rank_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t
     uint32_t wmax = 0, wmin = 0xFFFFFFFFu;
     unsigned long long wsum = 0;
     for (uint64_t p = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; p < n; p += warps) {
-        const uint32_t v = vert_at[p];
+        const uint32_t v = vert_at ? vert_at[p] : uint32_t(p);
         const uint64_t a = row[v], b = row[v + 1], o = nrow[p];
         for (uint64_t e = a + lane; e < b; e += 32) {
             const uint32_t wt = w[e];
-            arc[o + (e - a)] = make_uint2(pos_of[col[e]], wt);
+            arc[o + (e - a)] = make_uint2(vert_at ? pos_of[col[e]] : col[e], wt);
             wmax = max(wmax, wt);
             wmin = min(wmin, wt);
             wsum += wt;
@@ -267,16 +274,26 @@ int grid_for(uint64_t work, int tpb) {
         }                                                                       \
     } while (0)
 
+// A graph with short rows keeps the caller's numbering where neighbours are this
+// close in it, as a share of the vertices, on average (a grid by rows: 0.001;
+// by rank, or at random: a third): the vertices that a tree reaches then lie
+// together, and the slots' keys stay in the last level cache (grids of 262,000
+// vertices: 143 ms by rank, 127 ms so; 90,000: 33.5 and 32.1; 49,000 and fewer:
+// within 1%, the rank order stays). Scale-free graphs gain more from the rank
+// order, which puts the hubs together.
+static constexpr double LOCAL_GAP = 1.0 / 16;
+static constexpr uint32_t LOCAL_N = 65536;
+
 chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uint32_t *col,
-                         const uint32_t *w, const uint32_t *rank, RankGraph &g, cudaStream_t s,
+                         const uint32_t *w, const uint32_t *rank, bool keep_ids, RankGraph &g, cudaStream_t s,
                          int *launches) {
     chl_status st = CHL_OK;
     Check *chk = nullptr;
-    Check hchk{0, 0, 0};
+    Check hchk{};
     uint32_t *cnt = nullptr;
     uint64_t *deg = nullptr;
     WStats *ws = nullptr;
-    WStats hws{0, 0xFFFFFFFFu, 0, 0};
+    WStats hws{0, 0xFFFFFFFFu, 0};
     g = RankGraph{};
     g.n = n;
     g.m2 = m2;
@@ -330,11 +347,17 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(dmalloc(&g.arc, (m2 ? m2 : 1) * sizeof(uint2), s));
     CK(dmalloc(&ws, sizeof(WStats), s));
     CK(cudaMemcpyAsync(ws, &hws, sizeof(WStats), cudaMemcpyHostToDevice, s));
-    rank_degree_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, row, g.vert_at, deg, ws);
-    *launches += 1;
-    CK(cudaMemsetAsync(deg + n, 0, sizeof(uint64_t), s));
-    CK(exclusive_scan_u64(deg, g.row, uint64_t(n) + 1, s, launches));
-    rank_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, g.vert_at,
+    g.deg_max = hchk.deg_max;
+    g.caller_ids = keep_ids && n >= LOCAL_N && m2 && g.deg_max <= DIRECT_DEGREE && double(hchk.gap) / double(m2) < double(n) * LOCAL_GAP;
+    if (g.caller_ids) {
+        CK(cudaMemcpyAsync(g.row, row, (size_t(n) + 1) * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+    } else {
+        rank_degree_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, row, g.vert_at, deg);
+        *launches += 1;
+        CK(cudaMemsetAsync(deg + n, 0, sizeof(uint64_t), s));
+        CK(exclusive_scan_u64(deg, g.row, uint64_t(n) + 1, s, launches));
+    }
+    rank_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, g.caller_ids ? nullptr : g.vert_at,
                                                                      g.pos_of, g.row, g.arc, ws);
     *launches += 1;
     CK(cudaGetLastError());
@@ -342,7 +365,6 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(cudaStreamSynchronize(s));
     g.w_max = m2 ? hws.wmax : 1;
     g.w_min = m2 ? hws.wmin : 1;
-    g.deg_max = hws.dmax;
     g.w_mean = m2 ? double(hws.wsum) / double(m2) : 1.0;
 done:
     if (chk) cudaFreeAsync(chk, s);

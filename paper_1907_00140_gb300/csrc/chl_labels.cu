@@ -34,10 +34,10 @@ __global__ void count_kernel(uint64_t T, const uint32_t *v, uint64_t *cnt) {
 // vertex's segment; records of hubs below min_hub are left out (the dense
 // Common Label Table answers for those hubs)
 __global__ void count_table_kernel(uint64_t T, const uint32_t *v, const uint32_t *h,
-                                   const uint32_t *pos_of, uint32_t min_hub, uint64_t *cnt) {
+                                   const uint32_t *index_of, uint32_t min_hub, uint64_t *cnt) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < T;
          i += uint64_t(gridDim.x) * blockDim.x)
-        if (h[i] >= min_hub) atomicAdd((unsigned long long *)&cnt[pos_of[v[i]]], 1ull);
+        if (h[i] >= min_hub) atomicAdd((unsigned long long *)&cnt[index_of ? index_of[v[i]] : v[i]], 1ull);
 }
 
 // the entries of a label table in either form
@@ -58,12 +58,12 @@ struct TableEntries {
 };
 
 __global__ void scatter_table_kernel(uint64_t T, const uint32_t *v, const uint32_t *h,
-                                     const uint32_t *d, const uint32_t *pos_of, uint32_t min_hub,
+                                     const uint32_t *d, const uint32_t *index_of, uint32_t min_hub,
                                      const uint64_t *off, uint64_t *fill, TableEntries e) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < T;
          i += uint64_t(gridDim.x) * blockDim.x) {
         if (h[i] < min_hub) continue;
-        const uint32_t x = pos_of[v[i]];
+        const uint32_t x = index_of ? index_of[v[i]] : v[i];
         const uint64_t k = off[x] + atomicAdd((unsigned long long *)&fill[x], 1ull);
         e.put(k, h[i], d[i]);
     }
@@ -92,13 +92,13 @@ __global__ void copy_segments_kernel(uint32_t n, const uint64_t *old_off, TableE
 
 // new records after each vertex's old entries
 __global__ void scatter_new_kernel(uint64_t T0, uint64_t T, const uint32_t *v, const uint32_t *h,
-                                   const uint32_t *d, const uint32_t *pos_of, uint32_t min_hub,
+                                   const uint32_t *d, const uint32_t *index_of, uint32_t min_hub,
                                    const uint64_t *old_off, const uint64_t *off, uint64_t *fill,
                                    TableEntries e) {
     for (uint64_t i = T0 + uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < T;
          i += uint64_t(gridDim.x) * blockDim.x) {
         if (h[i] < min_hub) continue;
-        const uint32_t x = pos_of[v[i]];
+        const uint32_t x = index_of ? index_of[v[i]] : v[i];
         const uint64_t k = off[x] + (old_off[x + 1] - old_off[x]) +
                            atomicAdd((unsigned long long *)&fill[x], 1ull);
         e.put(k, h[i], d[i]);
@@ -461,7 +461,7 @@ static cudaError_t alloc_entries(LabelTable &t, uint64_t T, int db, cudaStream_t
 // Entries are allocated with two spare ones past the last, so that a read
 // widened to 16-byte boundaries (two entries) stays inside the array.
 cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const uint32_t *in_h,
-                           const uint32_t *in_d, const uint32_t *pos_of, uint32_t min_hub,
+                           const uint32_t *in_d, const uint32_t *index_of, uint32_t min_hub,
                            int db, LabelTable &out, cudaStream_t s, int *launches) {
     cudaError_t e = cudaSuccess;
     uint64_t *cnt = nullptr;
@@ -470,12 +470,12 @@ cudaError_t assemble_table(uint32_t n, uint64_t T, const uint32_t *in_v, const u
     CKE(alloc_entries(out, T, db, s));
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
-    count_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, pos_of, min_hub, cnt);
+    count_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, index_of, min_hub, cnt);
     *launches += 1;
     CKE(cudaGetLastError());
     CKE(exclusive_scan_u64(cnt, out.offsets, uint64_t(n) + 1, s, launches));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
-    scatter_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, in_d, pos_of, min_hub,
+    scatter_table_kernel<<<grid_for(T, 256), 256, 0, s>>>(T, in_v, in_h, in_d, index_of, min_hub,
                                                           out.offsets, cnt, TableEntries(out));
     *launches += 1;
     CKE(cudaGetLastError());
@@ -488,7 +488,7 @@ done:
 }
 
 cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, const uint32_t *in_v,
-                       const uint32_t *in_h, const uint32_t *in_d, const uint32_t *pos_of,
+                       const uint32_t *in_h, const uint32_t *in_d, const uint32_t *index_of,
                        uint32_t min_hub, int db, cudaStream_t s, int *launches, LabelTable *keep_old) {
     cudaError_t e = cudaSuccess;
     uint64_t *cnt = nullptr;
@@ -499,7 +499,7 @@ cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, cons
     CKE(dmalloc(&cnt, (size_t(n) + 1) * sizeof(uint64_t), s));
     CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
     if (dT) {
-        count_table_kernel<<<grid_for(dT, 256), 256, 0, s>>>(dT, in_v + T0, in_h + T0, pos_of, min_hub,
+        count_table_kernel<<<grid_for(dT, 256), 256, 0, s>>>(dT, in_v + T0, in_h + T0, index_of, min_hub,
                                                              cnt);
         *launches += 1;
     }
@@ -513,7 +513,7 @@ cudaError_t grow_table(uint32_t n, LabelTable &lt, uint64_t T0, uint64_t T, cons
     CKE(cudaGetLastError());
     if (dT) {
         CKE(cudaMemsetAsync(cnt, 0, (size_t(n) + 1) * sizeof(uint64_t), s));
-        scatter_new_kernel<<<grid_for(dT, 256), 256, 0, s>>>(T0, T, in_v, in_h, in_d, pos_of, min_hub,
+        scatter_new_kernel<<<grid_for(dT, 256), 256, 0, s>>>(T0, T, in_v, in_h, in_d, index_of, min_hub,
                                                              lt.offsets, out.offsets, cnt, TableEntries(out));
         *launches += 1;
         CKE(cudaGetLastError());

@@ -216,15 +216,16 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         __syncthreads();
         const uint32_t h = S.root;
         if (h == NONE) break;
+        const uint32_t hv = root_vertex<K>(p, h);
         // the pruning tables of the root (see chl_tree.cu)
         const bool prune = p.hc && h >= p.hc_hubs;
         if (prune)
-            for (uint32_t k = tid; k < p.hc_stride; k += TPB) S.hch[k] = __ldg(&p.hc[size_t(h) * p.hc_stride + k]);
+            for (uint32_t k = tid; k < p.hc_stride; k += TPB) S.hch[k] = __ldg(&p.hc[size_t(hv) * p.hc_stride + k]);
         const bool lt = p.lt_off && h >= p.lt_hubs;
         bool fits = true;
         if (lt) {
-            const uint64_t a = __ldg(&p.lt_off[h]);
-            const uint32_t cnt = uint32_t(__ldg(&p.lt_off[h + 1]) - a);
+            const uint64_t a = __ldg(&p.lt_off[hv]);
+            const uint32_t cnt = uint32_t(__ldg(&p.lt_off[hv + 1]) - a);
             fits = cnt <= LTH_MAX;
             if (fits) {
                 for (uint32_t i = tid; i < LTH_SLOTS; i += TPB) S.lth_key[i] = 0;
@@ -245,8 +246,8 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         if (fits) {
             if (tid == 0) {
                 constexpr int BITS = 31 - __builtin_clz(SLOTS);
-                const uint32_t s = (h * 2654435761u) >> (32 - BITS);
-                S.id[s] = h | PENDING;
+                const uint32_t s = (hv * 2654435761u) >> (32 - BITS);
+                S.id[s] = hv | PENDING;
                 S.key[s] = make_key<K>(0, true, h);
                 S.touch[0] = uint16_t(s);
                 S.n_touch = 1;
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                         s = S.pend[x][i];
                         const KS k = S.key[s];
                         const uint32_t v = S.id[s] & ID_MASK, d = key_dist<K>(k);
-                        live |= is_live<K>(k, v, h);
+                        live |= is_live<K>(k, pos_at<K>(p, v), h);
                         in = d < t_hi;
                         keep = !in;
                         if (in) S.id[s] = v;  // no longer pending
@@ -301,7 +302,8 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                         const uint64_t rs = __ldg(&p.row[v]);
                         deg = uint32_t(__ldg(&p.row[v + 1]) - rs);
                         S.rs[tid] = rs;
-                        S.kv[tid] = make_key<K>(dv, is_live<K>(k, v, h), v);
+                        const uint32_t vpos = pos_at<K>(p, v);
+                        S.kv[tid] = make_key<K>(dv, is_live<K>(k, vpos, h), vpos);
                         if (lt) {
                             const uint64_t a = __ldg(&p.lt_off[v]);
                             len = uint32_t(__ldg(&p.lt_off[v + 1]) - a);
@@ -310,7 +312,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                         }
                         cut = prune && clt_prunes(p, S, v, dv);
                         if (lt) {
-                            cut |= v < p.lt_hubs;  // a table hub: the complete query would prune it
+                            cut |= vpos < p.lt_hubs;  // a table hub: the complete query would prune it
                             if (cut) len = 0;
                             S.len[tid] = len;
                         }
@@ -386,7 +388,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         for (uint32_t i = tid; i < nt; i += TPB) {
             const uint32_t s = S.touch[i];
             const KS k = S.key[s];
-            const bool on = is_live<K>(k, S.id[s] & ID_MASK, h);
+            const bool on = is_live<K>(k, pos_at<K>(p, S.id[s] & ID_MASK), h);
             mine += on;
             if (on) far = max(far, key_dist<K>(k));
         }
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                 const uint32_t s = S.touch[i];
                 v = S.id[s] & ID_MASK;
                 k = S.key[s];
-                on = ok && is_live<K>(k, v, h);
+                on = ok && is_live<K>(k, pos_at<K>(p, v), h);
                 S.id[s] = EMPTY;
                 S.key[s] = key_inf<K>();
             }
@@ -431,7 +433,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
             if (lane == 0) at = atomicAdd(&S.n_put, uint32_t(__popc(m)));
             at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << lane) - 1));
             if (on) {
-                p.out_v[base + at] = __ldg(&p.vert_at[v]);
+                p.out_v[base + at] = caller_id<K>(p, v);
                 p.out_h[base + at] = h;
                 p.out_d[base + at] = key_dist<K>(k);
                 if (p.out_p) p.out_p[base + at] = __ldg(&p.vert_at[key_parent<K>(k)]);
@@ -472,6 +474,10 @@ cudaError_t launch_class(const TreeLaunch &p, uint32_t max_trees, uint32_t *spil
 template <int TPB, int SLOTS>
 cudaError_t launch_key(const TreeLaunch &p, uint32_t max_trees, uint32_t *spill, unsigned int *spill_n,
                        cudaStream_t s) {
+    if (p.pos)
+        return p.out_p            ? launch_class<TPB, SLOTS, ById<KeyP>>(p, max_trees, spill, spill_n, s)
+               : p.key_bytes == 4 ? launch_class<TPB, SLOTS, ById<KeyN>>(p, max_trees, spill, spill_n, s)
+                                  : launch_class<TPB, SLOTS, ById<KeyW>>(p, max_trees, spill, spill_n, s);
     if (p.out_p) return launch_class<TPB, SLOTS, KeyP>(p, max_trees, spill, spill_n, s);
     if (p.key_bytes == 4) return launch_class<TPB, SLOTS, KeyN>(p, max_trees, spill, spill_n, s);
     return launch_class<TPB, SLOTS, KeyW>(p, max_trees, spill, spill_n, s);

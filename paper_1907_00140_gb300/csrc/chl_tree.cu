@@ -304,8 +304,9 @@ __device__ __forceinline__ void commit_one(const TreeLaunch &p, Shared &S, const
         const bool unreached = old == key_inf<K>();
         const uint32_t nb = bucket_of(p, key_dist<K>(cand));
         const uint32_t ob = unreached ? NONE : bucket_of(p, key_dist<K>(old));
-        const bool f_new = nb > S.bcur && is_live<K>(cand, u, h);
-        const bool f_old = !unreached && ob > S.bcur && is_live<K>(old, u, h);
+        const uint32_t pu = pos_at<K>(p, u);
+        const bool f_new = nb > S.bcur && is_live<K>(cand, pu, h);
+        const bool f_old = !unreached && ob > S.bcur && is_live<K>(old, pu, h);
         dcnt = int(f_new) - int(f_old);
         if (nb == S.bcur) {
             if (atomicExch(&sl.rtag[u], S.rid) != S.rid) cls = 1;
@@ -587,7 +588,7 @@ __device__ void lt_answer(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F, u
 template <int TPB, typename K>
 __device__ __forceinline__ void direct_pass(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F,
                                             const Slot<K> &sl, uint32_t h, uint64_t rs, uint32_t deg,
-                                            uint32_t dv, bool lv, uint32_t vid) {
+                                            uint32_t dv, bool lv, uint32_t vpos) {
     using KS = typename K::T;
     const int lane = threadIdx.x & 31;
     // the keys of a list that is counted on entry are all read before any
@@ -595,7 +596,7 @@ __device__ __forceinline__ void direct_pass(const TreeLaunch &p, Shared &S, Fron
     if (S.fuse_live || S.lt_prune) __syncthreads();
     const uint32_t most = __reduce_max_sync(FULL, deg), arcs = __reduce_add_sync(FULL, deg);
     if (lane == 0) F.n_arcs[threadIdx.x >> 5] += arcs;
-    const KS kv = make_key<K>(dv, lv, vid);
+    const KS kv = make_key<K>(dv, lv, vpos);
     uint32_t bn = 0;  // improvements in the warp's buffer
     for (uint32_t e = 0; e < most; e += K::U) {
         uint2 a[K::U];
@@ -637,17 +638,18 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
         const uint32_t *cur = S.cur_slot != NONE ? sl.sub(S.cur_slot) : (S.sel ? sl.l1() : sl.l0());
         const uint32_t i = cb + threadIdx.x;
         uint64_t deg = 0, rs = 0;
-        uint32_t dv = 0, vid = 0;
+        uint32_t dv = 0, vid = 0, vpos = 0;
         bool lv = false, clean = false, cut = false, ask = false, ex = false;
         if (i < n_cur) {
             const uint32_t v = cur[i];
             const KS k = __ldcg(&sl.key[v]);
             vid = v;
+            vpos = pos_at<K>(p, v);
             if (key_dist<K>(k) >= t_lo) {  // else stale: expanded in an earlier bucket
                 dv = key_dist<K>(k);
                 rs = __ldg(&p.row[v]);
                 deg = __ldg(&p.row[v + 1]) - rs;
-                lv = is_live<K>(k, v, h);
+                lv = is_live<K>(k, vpos, h);
                 clean = key_clean<K>(k);
                 if (v < p.fin_bits && uint64_t(dv) < t_lo + p.w_min)
                     atomicOr(&fin_bitmap[v >> 5], 1u << (v & 31));
@@ -657,7 +659,7 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
                 // their shortest paths, which outranks v and so is a table hub
                 // too: the complete query would find it
                 if (!cut && S.lt_prune) {
-                    if (v < p.lt_hubs) cut = true;
+                    if (vpos < p.lt_hubs) cut = true;
                     else ask = true;
                 }
             }
@@ -709,7 +711,7 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
             if (lane == 0 && c) atomicSub(&S.cnt, c);
         }
         if (p.direct) {
-            direct_pass<TPB, K>(p, S, F, sl, h, rs, uint32_t(deg), dv, lv, vid);
+            direct_pass<TPB, K>(p, S, F, sl, h, rs, uint32_t(deg), dv, lv, vpos);
             continue;
         }
         const bool ok = deg != 0;
@@ -746,7 +748,7 @@ __device__ void expand_round(const TreeLaunch &p, Shared &S, Frontier<TPB, K> &F
             const uint32_t c = rl + __popc(okm & ((1u << lane) - 1));
             const uint64_t pre = dl + inc - deg;
             F.base[c] = rs - pre;  // wraps: base + position = rs + (position - pre)
-            F.kv[c] = make_key<K>(dv, lv, vid);
+            F.kv[c] = make_key<K>(dv, lv, vpos);
             F.pre[c] = pre;
         }
         const uint64_t total = da;
@@ -893,7 +895,7 @@ __device__ void count_live_in_bucket(const TreeLaunch &p, Shared &S, const Slot<
     for (uint32_t i = threadIdx.x; i < cnt; i += TPB) {
         const uint32_t u = lst[i];
         const typename K::T k = __ldcg(&sl.key[u]);
-        c += (bucket_of(p, key_dist<K>(k)) == b && is_live<K>(k, u, h));
+        c += (bucket_of(p, key_dist<K>(k)) == b && is_live<K>(k, pos_at<K>(p, u), h));
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
@@ -961,13 +963,14 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
         const uint32_t h = S.root;
         if (h == NONE) break;
         if (threadIdx.x == 0) ++S.n_trees;
+        const uint32_t hv = root_vertex<K>(p, h);
 
         // trivial tree: every neighbour outranks the root, so after the root is
         // popped no queued vertex has the root as ancestor (cnt = 0)
         bool lower = false;
         {
-            const uint64_t rs = p.row[h], re = p.row[h + 1];
-            for (uint64_t e = rs + threadIdx.x; e < re; e += TPB) lower |= (__ldg(&p.arc[e]).x > h);
+            const uint64_t rs = p.row[hv], re = p.row[hv + 1];
+            for (uint64_t e = rs + threadIdx.x; e < re; e += TPB) lower |= pos_at<K>(p, __ldg(&p.arc[e]).x) > h;
         }
         const bool nontrivial = __syncthreads_or(lower);
 
@@ -976,7 +979,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
             if (threadIdx.x == 0) ++S.n_trivial;
             if (threadIdx.x == 0) {
                 S.out_n = 1;
-                sl.l0()[0] = h;
+                sl.l0()[0] = hv;
                 sl.l1()[0] = 0;
                 sl.far()[0] = h;  // the root is its own parent
             }
@@ -991,7 +994,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
             const bool prune = p.hc && h >= p.hc_hubs;
             if (prune)
                 for (uint32_t c = threadIdx.x; c < p.hc_stride; c += TPB)
-                    S.hch[c] = __ldg(&p.hc[size_t(h) * p.hc_stride + c]);
+                    S.hch[c] = __ldg(&p.hc[size_t(hv) * p.hc_stride + c]);
             if (threadIdx.x == 0) S.prune = prune;
             // the label table of earlier phases: the root's labels in it, as
             // distances by hub position in shared memory when the table's hubs
@@ -1002,8 +1005,8 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
             const bool lt_shared = lt_prune && !p.stage_bytes && p.lt_hubs <= p.aux_bytes / 4;
             uint64_t lt_a = 0, lt_b = 0;
             if (lt_prune) {
-                lt_a = __ldg(&p.lt_off[h]);
-                lt_b = __ldg(&p.lt_off[h + 1]);
+                lt_a = __ldg(&p.lt_off[hv]);
+                lt_b = __ldg(&p.lt_off[hv + 1]);
                 lt_dense = !lt_shared && lt_b - lt_a > min(LTH_MAX, p.lt_hash_max);  // uniform over the CTA
                 lt_prune = !lt_dense || p.lt_root;
                 lt_dense = lt_dense && lt_prune;
@@ -1060,9 +1063,9 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                 S.abort = 0;
                 S.fuse_live = 0;
                 S.qn = 0;
-                sl.l0()[0] = h;
-                sl.touch()[0] = h;
-                atomic_set_key(&sl.key[h], make_key<K>(0, true, h));
+                sl.l0()[0] = hv;
+                sl.touch()[0] = hv;
+                atomic_set_key(&sl.key[hv], make_key<K>(0, true, h));
             }
             __syncthreads();
             uint32_t rounds = 0;
@@ -1161,7 +1164,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
                 if (i < nt) {
                     u = sl.touch()[i];
                     const typename K::T k = __ldcg(&sl.key[u]);
-                    lv = is_live<K>(k, u, h);
+                    lv = is_live<K>(k, pos_at<K>(p, u), h);
                     d = key_dist<K>(k);
                     par = key_parent<K>(k);
                     if (lv) far = max(far, d);
@@ -1209,7 +1212,7 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
         if (S.ok) {
             const unsigned long long b = S.base;
             for (uint32_t i = threadIdx.x; i < nlab; i += TPB) {
-                p.out_v[b + i] = __ldg(&p.vert_at[sl.l0()[i]]);
+                p.out_v[b + i] = caller_id<K>(p, sl.l0()[i]);
                 p.out_h[b + i] = h;
                 p.out_d[b + i] = sl.l1()[i];
                 if (p.out_p) p.out_p[b + i] = __ldg(&p.vert_at[sl.far()[i]]);
@@ -1267,11 +1270,30 @@ size_t dyn_bytes(uint32_t fin_words, uint32_t aux_bytes) {
     return aux_bytes ? ((size_t(fin_words) * 4 + 127) & ~size_t(127)) + aux_bytes : size_t(fin_words) * 4;
 }
 
+// the kernels of graphs in the caller's numbering
+template <int TPB, typename K>
+cudaError_t launch_ids(const TreeLaunch &p, int slots, size_t smem, cudaStream_t s) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (!e) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, ById<K>>, optin);
+    if (e) return e;
+    plant_trees_kernel<TPB, ById<K>><<<slots, TPB, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
 template <int TPB>
 cudaError_t launch_t(const TreeLaunch &p, int slots, cudaStream_t s) {
     cudaError_t e = allow_smem<TPB>();
     if (e) return e;
     const size_t smem = dyn_bytes(p.fin_words, p.aux_bytes);
+    if (p.pos) {
+        if constexpr (caller_ids_block(TPB))
+            return p.out_p            ? launch_ids<TPB, KeyP>(p, slots, smem, s)
+                   : p.key_bytes == 4 ? launch_ids<TPB, KeyN>(p, slots, smem, s)
+                                      : launch_ids<TPB, KeyW>(p, slots, smem, s);
+        return cudaErrorInvalidValue;
+    }
     if (p.out_p)
         plant_trees_kernel<TPB, KeyP><<<slots, TPB, smem, s>>>(p);
     else if (p.key_bytes == 4)
@@ -1398,24 +1420,24 @@ namespace {
 // Common Label Table from label records: record i is (caller vertex out_v[i],
 // hub pos out_h[i], distance out_d[i]); those of hubs below `hubs` go in
 __global__ void clt_fill_kernel(const uint32_t *out_v, const uint32_t *out_h, const uint32_t *out_d,
-                                unsigned long long count, const uint32_t *pos_of, uint32_t *hc,
+                                unsigned long long count, const uint32_t *index_of, uint32_t *hc,
                                 uint32_t stride, uint32_t hubs) {
     for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < count;
          i += (unsigned long long)gridDim.x * blockDim.x) {
         const uint32_t c = out_h[i];
-        if (c < hubs) hc[size_t(pos_of[out_v[i]]) * stride + c] = out_d[i];
+        if (c < hubs) hc[size_t(index_of ? index_of[out_v[i]] : out_v[i]) * stride + c] = out_d[i];
     }
 }
 
 }  // namespace
 
 cudaError_t launch_clt_fill(const uint32_t *out_v, const uint32_t *out_h, const uint32_t *out_d,
-                            unsigned long long count, const uint32_t *pos_of, uint32_t *hc,
+                            unsigned long long count, const uint32_t *index_of, uint32_t *hc,
                             uint32_t stride, uint32_t hubs, cudaStream_t s) {
     if (!count) return cudaSuccess;
     unsigned long long blocks = (count + 255) / 256;
     if (blocks > uint64_t(device_sms()) * 32) blocks = uint64_t(device_sms()) * 32;
-    clt_fill_kernel<<<unsigned(blocks), 256, 0, s>>>(out_v, out_h, out_d, count, pos_of, hc, stride,
+    clt_fill_kernel<<<unsigned(blocks), 256, 0, s>>>(out_v, out_h, out_d, count, index_of, hc, stride,
                                                      hubs);
     return cudaGetLastError();
 }
@@ -1435,8 +1457,12 @@ __global__ void split_trivial_kernel(TreeLaunch p, uint32_t begin, uint32_t coun
     const uint32_t h = begin + i;
     if (i < count) {
         triv = true;
-        const uint64_t rs = __ldg(&p.row[h]), re = __ldg(&p.row[h + 1]);
-        for (uint64_t e = rs; e < re && triv; ++e) triv = __ldg(&p.arc[e]).x <= h;
+        const uint32_t hv = p.pos ? __ldg(&p.vert_at[h]) : h;
+        const uint64_t rs = __ldg(&p.row[hv]), re = __ldg(&p.row[hv + 1]);
+        for (uint64_t e = rs; e < re && triv; ++e) {
+            const uint32_t u = __ldg(&p.arc[e]).x;
+            triv = (p.pos ? __ldg(&p.pos[u]) : u) <= h;
+        }
     }
     const unsigned tm = __ballot_sync(0xffffffffu, triv);
     const unsigned om = __ballot_sync(0xffffffffu, i < count && !triv);

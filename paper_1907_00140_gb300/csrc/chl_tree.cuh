@@ -42,9 +42,16 @@ constexpr int QSTEPS = 4;             // label-table query from global memory: l
 // U: arcs a lane relaxes per step of the arc pass (its loads in flight); the
 // 8-byte layouts take two, so that a thread's probe state fits its registers
 // at 1024 threads per SM.
-struct KeyN { using T = uint32_t; static constexpr int S = 1; static constexpr int U = 4; };
-struct KeyW { using T = uint64_t; static constexpr int S = 1; static constexpr int U = 2; };
-struct KeyP { using T = uint64_t; static constexpr int S = 32; static constexpr int U = 2; };
+// IDS: vertices are numbered as by the caller and their rank positions read from
+// p.pos (a type of its own, so that the kernels of rank-ordered graphs pay
+// nothing for it).
+struct KeyN { using T = uint32_t; static constexpr int S = 1; static constexpr int U = 4; static constexpr bool IDS = false; };
+struct KeyW { using T = uint64_t; static constexpr int S = 1; static constexpr int U = 2; static constexpr bool IDS = false; };
+struct KeyP { using T = uint64_t; static constexpr int S = 32; static constexpr int U = 2; static constexpr bool IDS = false; };
+template <typename K>
+struct ById : K {
+    static constexpr bool IDS = true;
+};
 
 template <typename K>
 __device__ __forceinline__ typename K::T key_inf() { return ~typename K::T(0); }
@@ -67,14 +74,23 @@ __device__ __forceinline__ uint64_t key_dist_limit() {
     return sizeof(typename K::T) == 4 ? 0x7FFFFFFEull : 0xFFFFFFFEull;
 }
 
+// rank position of a vertex; caller's id of a vertex; vertex of a root (given by
+// its rank position)
+template <typename K>
+__device__ __forceinline__ uint32_t pos_at(const TreeLaunch &p, uint32_t v) { return K::IDS ? __ldg(&p.pos[v]) : v; }
+template <typename K>
+__device__ __forceinline__ uint32_t caller_id(const TreeLaunch &p, uint32_t v) { return K::IDS ? v : __ldg(&p.vert_at[v]); }
+template <typename K>
+__device__ __forceinline__ uint32_t root_vertex(const TreeLaunch &p, uint32_t h) { return K::IDS ? __ldg(&p.vert_at[h]) : h; }
+
 // bucket of a distance: a shift when the width is a power of two
 __device__ __forceinline__ uint32_t bucket_of(const TreeLaunch &p, uint32_t d) {
     return p.delta_shift >= 0 ? d >> p.delta_shift : d / p.delta;
 }
 
 template <typename K>
-__device__ __forceinline__ bool is_live(typename K::T k, uint32_t v, uint32_t h) {
-    return key_clean<K>(k) && v >= h;
+__device__ __forceinline__ bool is_live(typename K::T k, uint32_t vpos, uint32_t h) {
+    return key_clean<K>(k) && vpos >= h;
 }
 
 __device__ __forceinline__ uint32_t atomic_min_key(uint32_t *a, uint32_t v) { return atomicMin(a, v); }

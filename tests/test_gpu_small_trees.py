@@ -39,7 +39,7 @@ def line_and_triples(line, triples, seed):
 
 def case(name):
     if name == "line":
-        return line_and_triples(1500, 14000, seed=4)
+        return line_and_triples(1500, 22000, seed=4)  # keeps its numbering, prunes by labels
     if name == "ba40k":
         g = W.barabasi_albert(40000, 2, seed=9, wlo=1, whi=100)
         return g, W.degree_rank(g)
@@ -67,7 +67,7 @@ def test_small_trees_equal_oracle(built, opts, capfd, monkeypatch):
     seen = [(int(c), int(s)) for c, s in re.findall(r"class (-?\d+) spilled (\d+)", capfd.readouterr().err)]
     assert_same(ref, *L.to_numpy())
     assert any(c >= 0 for c, _ in seen), seen  # the shared-memory kernel ran (its class depends on tree sizes)
-    if name == "line":
+    if name == "line" and "label_capacity" not in opts:  # (a phase built again reports its last attempt)
         assert any(s > 100 for _, s in seen), seen
     if opts.get("flags") == chl.CHL_FLAG_PARENTS and name == "line":
         off, hub, _ = L.to_numpy()
