@@ -46,6 +46,7 @@
 // (no partial tree is kept); the host rebuilds those roots after growing the
 // buffer.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 
 #include "chl_common.cuh"
@@ -1243,24 +1244,24 @@ __global__ void __launch_bounds__(TPB, TPB >= 64 ? 1024 / TPB : 16) plant_trees_
     }
 }
 
-// both key widths may take up to the opt-in maximum of dynamic shared memory
+// a kernel may take up to the opt-in maximum of dynamic shared memory (the
+// attribute belongs to the current device: set before every launch)
 template <typename F>
-cudaError_t allow_smem_of(F kernel, int optin) {
+cudaError_t allow_smem_of(F kernel) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (!e) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-    if (!e) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     optin - int(fa.sharedSizeBytes));
+    if (!e) e = cudaFuncGetAttributes(&fa, kernel);
+    if (!e) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - int(fa.sharedSizeBytes));
     return e;
 }
 
 template <int TPB>
 cudaError_t allow_smem() {
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (!e) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, KeyN>, optin);
-    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, KeyW>, optin);
-    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, KeyP>, optin);
+    cudaError_t e = allow_smem_of(plant_trees_kernel<TPB, KeyN>);
+    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, KeyW>);
+    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, KeyP>);
     return e;
 }
 
@@ -1270,39 +1271,27 @@ size_t dyn_bytes(uint32_t fin_words, uint32_t aux_bytes) {
     return aux_bytes ? ((size_t(fin_words) * 4 + 127) & ~size_t(127)) + aux_bytes : size_t(fin_words) * 4;
 }
 
-// the kernels of graphs in the caller's numbering
 template <int TPB, typename K>
-cudaError_t launch_ids(const TreeLaunch &p, int slots, size_t smem, cudaStream_t s) {
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (!e) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (!e) e = allow_smem_of(plant_trees_kernel<TPB, ById<K>>, optin);
+cudaError_t launch_k(const TreeLaunch &p, int slots, cudaStream_t s) {
+    const cudaError_t e = allow_smem_of(plant_trees_kernel<TPB, K>);
     if (e) return e;
-    plant_trees_kernel<TPB, ById<K>><<<slots, TPB, smem, s>>>(p);
+    plant_trees_kernel<TPB, K><<<slots, TPB, dyn_bytes(p.fin_words, p.aux_bytes), s>>>(p);
     return cudaGetLastError();
 }
 
 template <int TPB>
 cudaError_t launch_t(const TreeLaunch &p, int slots, cudaStream_t s) {
-    cudaError_t e = allow_smem<TPB>();
-    if (e) return e;
-    const size_t smem = dyn_bytes(p.fin_words, p.aux_bytes);
+    if (p.key_bytes != 4 && p.key_bytes != 8) return cudaErrorInvalidValue;
     if (p.pos) {
         if constexpr (caller_ids_block(TPB))
-            return p.out_p            ? launch_ids<TPB, KeyP>(p, slots, smem, s)
-                   : p.key_bytes == 4 ? launch_ids<TPB, KeyN>(p, slots, smem, s)
-                                      : launch_ids<TPB, KeyW>(p, slots, smem, s);
+            return p.out_p            ? launch_k<TPB, ById<KeyP>>(p, slots, s)
+                   : p.key_bytes == 4 ? launch_k<TPB, ById<KeyN>>(p, slots, s)
+                                      : launch_k<TPB, ById<KeyW>>(p, slots, s);
         return cudaErrorInvalidValue;
     }
-    if (p.out_p)
-        plant_trees_kernel<TPB, KeyP><<<slots, TPB, smem, s>>>(p);
-    else if (p.key_bytes == 4)
-        plant_trees_kernel<TPB, KeyN><<<slots, TPB, smem, s>>>(p);
-    else if (p.key_bytes == 8)
-        plant_trees_kernel<TPB, KeyW><<<slots, TPB, smem, s>>>(p);
-    else
-        return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    return p.out_p            ? launch_k<TPB, KeyP>(p, slots, s)
+           : p.key_bytes == 4 ? launch_k<TPB, KeyN>(p, slots, s)
+                              : launch_k<TPB, KeyW>(p, slots, s);
 }
 
 // CTAs per SM with `bytes` of dynamic shared memory; all key layouts are built
@@ -1330,7 +1319,7 @@ constexpr uint32_t SMEM_PER_SM_CAP = SMEM_CAP_BYTES;
 // the most dynamic shared memory (a multiple of 128 bytes) that keeps the
 // register-limited number of CTAs per SM, within SMEM_PER_SM_CAP per SM
 template <int TPB>
-uint32_t dyn_budget_t() {
+uint32_t dyn_budget_of() {
     const int full = occ<TPB>(0);
     if (full <= 0) return 0;
     int dev = 0, optin = 0;
@@ -1352,6 +1341,22 @@ uint32_t dyn_budget_t() {
     const int64_t cap = int64_t(SMEM_PER_SM_CAP) / full - int64_t(fa.sharedSizeBytes) - 1024;
     const uint32_t c = cap > 0 ? uint32_t(cap) & ~127u : 0u;
     return c < lo ? c : lo;
+}
+
+// a property of the device and the kernels (every phase of a build asks for it,
+// and the search takes dozens of occupancy queries): found once per device
+template <int TPB>
+uint32_t dyn_budget_t() {
+    constexpr int MAXDEV = 64;
+    static std::atomic<uint32_t> known[MAXDEV];  // budget + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAXDEV) return dyn_budget_of<TPB>();
+    uint32_t b = known[dev].load(std::memory_order_relaxed);
+    if (!b) {
+        b = dyn_budget_of<TPB>() + 1;
+        if (b > 1) known[dev].store(b, std::memory_order_relaxed);
+    }
+    return b - 1;
 }
 
 }  // namespace
