@@ -756,16 +756,6 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         d_w = (const uint32_t *)b_w.p;
         d_rank = (const uint32_t *)b_rank.p;
     }
-    {
-        uint64_t last = 0;
-        CUDA_TRY(cudaMemcpyAsync(&last, d_row + n, 8, cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-        if (last != m2) {
-            st = set_error(CHL_EINVAL, "row_ptr[n] = %llu differs from num_arcs = %llu",
-                           (unsigned long long)last, (unsigned long long)m2);
-            goto done;
-        }
-    }
     st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, keep_ids, rg, s, &launches);
     if (st != CHL_OK) goto done;
 

@@ -99,6 +99,8 @@ struct Check {
     uint32_t bits;
     uint32_t where;  // a vertex where the first failure was seen (any)
     uint32_t deg_max;  // longest row
+    uint32_t wmax, wmin;
+    unsigned long long wsum;
     unsigned long long gap; // sum of |u - v| over the arcs
     unsigned long long fp;  // symmetry fingerprint: sum of h(v, u, w) - h(u, v, w) over the arcs
 };
@@ -135,8 +137,14 @@ __device__ __forceinline__ unsigned long long arc_hash(uint32_t a, uint32_t b, u
 // with equal weights both ways, so the sum of h(v, u, w) - h(u, v, w) is 0
 // for every undirected graph; any other sum proves an arc without its
 // reverse, which check_symm_kernel then locates.
+// Weight statistics come from the same pass. Rows or ranks found bad by the
+// kernels before end it at once (its rows could lead anywhere), so that one
+// wait of the host sees every check.
 __global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t *col,
                                   const uint32_t *w, Check *c) {
+    if (*(volatile uint32_t *)&c->bits & (BAD_ROWPTR | BAD_RANK)) return;
+    uint32_t wmax = 0, wmin = 0xFFFFFFFFu;
+    unsigned long long wsum = 0;
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
     unsigned long long fp = 0, gap = 0;
@@ -149,6 +157,9 @@ __global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_
             if (u == v) fail(c, BAD_SELF, uint32_t(v));
             if (e > a && col[e - 1] >= u) fail(c, BAD_ORDER, uint32_t(v));
             gap += u > v ? u - v : v - u;
+            wmax = max(wmax, wt);
+            wmin = min(wmin, wt);
+            wsum += wt;
             fp += arc_hash(uint32_t(v), u, wt) - arc_hash(u, uint32_t(v), wt);
         }
     }
@@ -156,9 +167,17 @@ __global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_
     for (int o = 16; o; o >>= 1) {
         fp += __shfl_xor_sync(0xffffffffu, fp, o);
         gap += __shfl_xor_sync(0xffffffffu, gap, o);
+        wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
     }
+    wmax = __reduce_max_sync(0xffffffffu, wmax);
+    wmin = __reduce_min_sync(0xffffffffu, wmin);
     if (lane == 0 && fp) atomicAdd(&c->fp, fp);
-    if (lane == 0 && gap) atomicAdd(&c->gap, gap);
+    if (lane == 0 && wsum) {
+        atomicAdd(&c->gap, gap);
+        atomicAdd(&c->wsum, wsum);
+        atomicMax(&c->wmax, wmax);
+        atomicMin(&c->wmin, wmin);
+    }
 }
 
 // exact symmetry check, run only when the fingerprint is not 0: the reverse
@@ -208,11 +227,6 @@ __global__ void rank_perm_kernel(uint32_t n, const uint32_t *rank, const uint32_
     }
 }
 
-struct WStats {
-    uint32_t wmax, wmin;
-    unsigned long long wsum;
-};
-
 // degrees in rank order
 __global__ void rank_degree_kernel(uint32_t n, const uint64_t *row, const uint32_t *vert_at,
                                    uint64_t *deg) {
@@ -224,35 +238,18 @@ __global__ void rank_degree_kernel(uint32_t n, const uint64_t *row, const uint32
 }
 
 // one warp per vertex: copy its row with neighbours renumbered (vert_at null: as
-// they are), weight statistics
+// they are)
 __global__ void rank_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t *col,
                                  const uint32_t *w, const uint32_t *vert_at,
-                                 const uint32_t *pos_of, const uint64_t *nrow, uint2 *arc,
-                                 WStats *ws) {
+                                 const uint32_t *pos_of, const uint64_t *nrow, uint2 *arc) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    uint32_t wmax = 0, wmin = 0xFFFFFFFFu;
-    unsigned long long wsum = 0;
     for (uint64_t p = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; p < n; p += warps) {
         const uint32_t v = vert_at ? vert_at[p] : uint32_t(p);
         const uint64_t a = row[v], b = row[v + 1], o = nrow[p];
         for (uint64_t e = a + lane; e < b; e += 32) {
-            const uint32_t wt = w[e];
-            arc[o + (e - a)] = make_uint2(vert_at ? pos_of[col[e]] : col[e], wt);
-            wmax = max(wmax, wt);
-            wmin = min(wmin, wt);
-            wsum += wt;
+            arc[o + (e - a)] = make_uint2(vert_at ? pos_of[col[e]] : col[e], w[e]);
         }
-    }
-    for (int o = 16; o; o >>= 1) {
-        wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-        wmin = min(wmin, __shfl_xor_sync(0xffffffffu, wmin, o));
-        wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
-    }
-    if (lane == 0) {
-        atomicMax(&ws->wmax, wmax);
-        atomicMin(&ws->wmin, wmin);
-        atomicAdd(&ws->wsum, wsum);
     }
 }
 
@@ -292,13 +289,12 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     Check hchk{};
     uint32_t *cnt = nullptr;
     uint64_t *deg = nullptr;
-    WStats *ws = nullptr;
-    WStats hws{0, 0xFFFFFFFFu, 0};
     g = RankGraph{};
     g.n = n;
     g.m2 = m2;
     CK(dmalloc(&chk, sizeof(Check), s));
-    CK(cudaMemsetAsync(chk, 0, sizeof(Check), s));
+    hchk.wmin = 0xFFFFFFFFu;
+    CK(cudaMemcpyAsync(chk, &hchk, sizeof(Check), cudaMemcpyHostToDevice, s));
     CK(dmalloc(&cnt, size_t(n) * sizeof(uint32_t), s));
     CK(cudaMemsetAsync(cnt, 0, size_t(n) * sizeof(uint32_t), s));
     CK(dmalloc(&g.pos_of, size_t(n) * sizeof(uint32_t), s));
@@ -306,11 +302,20 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     check_rows_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, m2, row, chk);
     rank_count_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, rank, cnt, chk);
     rank_perm_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, rank, cnt, g.pos_of, g.vert_at, chk);
-    *launches += 3;
+    check_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, chk);
+    *launches += 4;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&hchk, chk, sizeof(Check), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (hchk.bits & BAD_ROWPTR) {
+        uint64_t last = 0;
+        CK(cudaMemcpyAsync(&last, row + n, sizeof(last), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (last != m2) {
+            st = set_error(CHL_EINVAL, "row_ptr[n] = %llu differs from num_arcs = %llu", (unsigned long long)last,
+                           (unsigned long long)m2);
+            goto done;
+        }
         st = set_error(CHL_EINVAL, "row_ptr is not a valid CSR offset array (vertex %u)", hchk.where);
         goto done;
     }
@@ -318,11 +323,6 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
         st = set_error(CHL_EINVAL, "rank is not a permutation of [0,n) (vertex %u)", hchk.where);
         goto done;
     }
-    check_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, chk);
-    *launches += 1;
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(&hchk, chk, sizeof(Check), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
     if (!(hchk.bits & BAD_COL) && hchk.fp) {
         // some arc has no reverse of equal weight: find a vertex that shows it
         check_symm_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, chk);
@@ -345,8 +345,6 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(dmalloc(&deg, (size_t(n) + 1) * sizeof(uint64_t), s));
     CK(dmalloc(&g.row, (size_t(n) + 1) * sizeof(uint64_t), s));
     CK(dmalloc(&g.arc, (m2 ? m2 : 1) * sizeof(uint2), s));
-    CK(dmalloc(&ws, sizeof(WStats), s));
-    CK(cudaMemcpyAsync(ws, &hws, sizeof(WStats), cudaMemcpyHostToDevice, s));
     g.deg_max = hchk.deg_max;
     g.caller_ids = keep_ids && n >= LOCAL_N && m2 && g.deg_max <= DIRECT_DEGREE && double(hchk.gap) / double(m2) < double(n) * LOCAL_GAP;
     if (g.caller_ids) {
@@ -358,19 +356,16 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
         CK(exclusive_scan_u64(deg, g.row, uint64_t(n) + 1, s, launches));
     }
     rank_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, g.caller_ids ? nullptr : g.vert_at,
-                                                                     g.pos_of, g.row, g.arc, ws);
+                                                                     g.pos_of, g.row, g.arc);
     *launches += 1;
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(&hws, ws, sizeof(WStats), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    g.w_max = m2 ? hws.wmax : 1;
-    g.w_min = m2 ? hws.wmin : 1;
-    g.w_mean = m2 ? double(hws.wsum) / double(m2) : 1.0;
+    g.w_max = m2 ? hchk.wmax : 1;
+    g.w_min = m2 ? hchk.wmin : 1;
+    g.w_mean = m2 ? double(hchk.wsum) / double(m2) : 1.0;
 done:
     if (chk) cudaFreeAsync(chk, s);
     if (cnt) cudaFreeAsync(cnt, s);
     if (deg) cudaFreeAsync(deg, s);
-    if (ws) cudaFreeAsync(ws, s);
     if (st != CHL_OK) free_graph(g, s);
     return st;
 }
