@@ -722,7 +722,6 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     bool overlap = false;
     bool listed = false;             // the current attempt runs from the device root list
     std::vector<uint32_t> list_h;    // ... whose host copy, when needed
-    uint32_t list_n = 0;
     // CHL_TRACE=1 prints one line per phase to stderr (host clock around the
     // stream synchronisations the build already makes)
     const bool trace = std::getenv("CHL_TRACE") && std::getenv("CHL_TRACE")[0] == '1';
@@ -932,11 +931,10 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         } else if (split) {
             CUDA_TRY(launch_split_trivial(tl, pb, pe - pb, (uint32_t *)b_roots.p, &ctl->list_n, s));
             ++launches;
-            CUDA_TRY(cudaMemcpyAsync(&list_n, &ctl->list_n, 4, cudaMemcpyDeviceToHost, s));
-            CUDA_TRY(cudaStreamSynchronize(s));
             tl.root_list = (const uint32_t *)b_roots.p;
             tl.root_begin = 0;
-            count = list_n;
+            tl.count_dev = &ctl->list_n;
+            count = pe - pb;  // a bound: the kernel reads the listed count, the host does not wait for it
             listed = true;
             list_h.clear();  // fetched if this attempt fails
         } else if (first) {
@@ -1063,6 +1061,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
             goto done;
         }
         T = records_kept(hc);
+        if (split) count = hc.list_n;
         std::vector<uint32_t> ffailed;  // the filler's trees that did not fit its buffer
         if (first && from_filler && !filler_merged) {
             // the filler's trees are this phase's too: wait for them, then take
