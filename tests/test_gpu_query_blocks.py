@@ -81,3 +81,30 @@ def test_long_side_of_a_path():
             want = list(range(u, v + 1)) if u <= v else list(range(u, v - 1, -1))
             assert int(lens[i]) == len(want)
             assert got[i, :min(len(want), max_len)].tolist() == want[:max_len]
+
+
+@pytest.mark.parametrize("mode", ["merge", "grouped", "parts"])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_pairs_are_read_in_stream_order(mode, pinned):
+    """Pairs in pinned memory that an earlier copy on the call's stream fills: the
+    call answers what the copy brings; pageable pairs give the same while the
+    stream is busy."""
+    g, rank, leaf = two_centres(40, 1, seed=4)
+    ref = O.build_labels(g, rank, "plant", threads=8)
+    pairs = np.random.default_rng(5).integers(0, g.n, (64, 2)).astype(np.uint32)
+    want = O.query(ref, rank, pairs)
+    assert (want != 0).any()
+    L = chl.build_labels(DG(g), dev(rank))
+    cut = [chl.build_labels(DG(g), dev(rank), root_begin=a, root_end=b) for a, b in ((0, 20), (20, g.n))]
+    src, big = dev(pairs), torch.randn(4096, 4096, device="cuda")
+    work = torch.cuda.Stream()
+    host = torch.zeros(64, 2, dtype=torch.int32, pin_memory=True)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(work):
+        for _ in range(20):
+            big @ big
+        host.copy_(src, non_blocking=True)
+    p = host.numpy().view(np.uint32) if pinned else pairs
+    got = (chl.query_partitioned(cut, p, stream=work.cuda_stream) if mode == "parts"
+           else L.query(p, stream=work.cuda_stream, grouped=mode == "grouped"))
+    assert np.array_equal(got, want)
