@@ -10,6 +10,7 @@
 // Algorithm 3 becomes an unsigned min inside the packed search key, and the
 // trees of the most important roots (the largest ones, Sec. 5.1 label counts
 // per tree) come first in the claim order.
+#include <algorithm>
 #include <cstdio>
 
 #include "chl_common.cuh"
@@ -118,7 +119,7 @@ __global__ void check_rows_kernel(uint32_t n, uint64_t m2, const uint64_t *row, 
         else dmax = max(dmax, b - a);
     }
     const uint32_t d = __reduce_max_sync(0xffffffffu, uint32_t(min(dmax, uint64_t(0xFFFFFFFFu))));
-    if ((threadIdx.x & 31) == 0 && d) atomicMax(&c->deg_max, d);
+    if ((threadIdx.x & 31) == 0 && d > *(volatile uint32_t *)&c->deg_max) atomicMax(&c->deg_max, d);
 }
 
 // 64-bit mix of an arc (the splitmix64 finaliser of Steele, Lea and Flood)
@@ -131,37 +132,103 @@ __device__ __forceinline__ unsigned long long arc_hash(uint32_t a, uint32_t b, u
     return x ^ (x >> 31);
 }
 
-// One warp per vertex: ids, weights, strictly increasing rows, no self-loop,
-// in one streaming pass. Symmetry by fingerprint: the arcs (v, u, w) form
+// The passes over the arcs give every warp an equal, contiguous piece of them,
+// whatever the rows: with a warp per row, one warp walked the longest row
+// (25,000 arcs of R-MAT scale 18) long after the others were done (builds with a warp
+// per row and so: scale 18 38.5 and 37.2 ms, scale 16 7.43 and 7.08 ms, 50,000
+// Barabasi-Albert vertices 9.75 and 9.55 ms; the rows are found with one search per
+// piece and 32 row ends a step after that).
+constexpr int ARC_TPB = 256;
+constexpr int ARC_STEP = 128;  // arcs of a warp in flight, four per lane
+constexpr int ARC_BLOCKS = 6;  // blocks per SM
+
+// the row that holds arc e < row[n]
+__device__ __forceinline__ uint32_t row_of(uint32_t n, const uint64_t *row, uint64_t e) {
+    uint32_t lo = 0, hi = n;  // row[lo] <= e < row[hi]
+    while (hi - lo > 1) {
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (row[mid] <= e) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// The row of arc e0 + min(lane, last) on each lane of a warp. v: a row at or
+// before that of e0, with no whole row of arcs between; on return the row of the
+// last of these arcs. 32 row ends a turn, looked up by shuffles.
+__device__ __forceinline__ uint32_t rows_of_step(uint32_t n, const uint64_t *row, uint64_t e0, uint32_t last,
+                                                 uint32_t &v) {
+    const uint32_t lane = threadIdx.x & 31, at = min(lane, last);
+    uint32_t r = 0;
+    bool found = false;
+    for (;;) {
+        const uint64_t i = uint64_t(v) + 1 + lane;
+        const uint32_t end = i <= n ? uint32_t(min(row[i] - e0, uint64_t(ARC_STEP))) : uint32_t(ARC_STEP);
+        uint32_t c = 0;  // row ends at or before the arc
+#pragma unroll
+        for (uint32_t o = 16; o; o >>= 1)
+            if (__shfl_sync(0xffffffffu, end, c + o - 1) <= at) c += o;
+        const uint32_t top = __shfl_sync(0xffffffffu, end, 31);
+        if (c == 31 && top <= at) c = 32;
+        if (!found && c < 32) {
+            r = v + c;
+            found = true;
+        }
+        if (top > last) break;
+        v += 32;
+    }
+    v = __shfl_sync(0xffffffffu, r, 31);
+    return r;
+}
+
+// Ids, weights, strictly increasing rows, no self-loop, in one streaming pass.
+// Symmetry by fingerprint: the arcs (v, u, w) form
 // the same multiset as their reverses (u, v, w) iff the graph is undirected
 // with equal weights both ways, so the sum of h(v, u, w) - h(u, v, w) is 0
 // for every undirected graph; any other sum proves an arc without its
 // reverse, which check_symm_kernel then locates.
 // Weight statistics come from the same pass. Rows or ranks found bad by the
 // kernels before end it at once (its rows could lead anywhere), so that one
-// wait of the host sees every check.
-__global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t *col,
-                                  const uint32_t *w, Check *c) {
+// wait of the host sees every check. One set of atomics per block (per warp, at
+// 39,000 warps, they queued up at their addresses).
+__global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
+    check_arcs_kernel(uint32_t n, uint64_t m2, uint64_t per_warp, const uint64_t *row, const uint32_t *col,
+                      const uint32_t *w, Check *c) {
     if (*(volatile uint32_t *)&c->bits & (BAD_ROWPTR | BAD_RANK)) return;
+    __shared__ unsigned long long part[3][ARC_TPB / 32];
+    __shared__ uint32_t most[ARC_TPB / 32], least[ARC_TPB / 32];
     uint32_t wmax = 0, wmin = 0xFFFFFFFFu;
     unsigned long long wsum = 0;
-    const int lane = threadIdx.x & 31;
-    const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long fp = 0, gap = 0;
-    for (uint64_t v = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-        const uint64_t a = row[v], b = row[v + 1];
-        for (uint64_t e = a + lane; e < b; e += 32) {
-            const uint32_t u = col[e], wt = w[e];
-            if (u >= n) { fail(c, BAD_COL, uint32_t(v)); continue; }
-            if (wt == 0) fail(c, BAD_WEIGHT, uint32_t(v));
-            if (u == v) fail(c, BAD_SELF, uint32_t(v));
-            if (e > a && col[e - 1] >= u) fail(c, BAD_ORDER, uint32_t(v));
+    const uint64_t lo = (uint64_t(blockIdx.x) * (ARC_TPB / 32) + warp) * per_warp, hi = min(lo + per_warp, m2);
+    uint32_t row0 = lo < hi ? row_of(n, row, lo) : 0;
+    for (uint64_t e0 = lo; e0 < hi; e0 += ARC_STEP) {
+        uint32_t nb[ARC_STEP / 32], we[ARC_STEP / 32];
+#pragma unroll
+        for (int k = 0; k < ARC_STEP / 32; ++k) {
+            const uint64_t e = e0 + 32 * k + lane;
+            nb[k] = e < hi ? col[e] : 0;
+            we[k] = e < hi ? w[e] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < ARC_STEP / 32; ++k) {
+            const uint64_t b = e0 + 32 * k, e = b + lane;
+            if (b >= hi) break;
+            const uint32_t v = rows_of_step(n, row, b, uint32_t(min(hi - b, uint64_t(32))) - 1, row0);
+            if (e >= hi) continue;
+            const uint32_t u = nb[k], wt = we[k];
+            if (u >= n) { fail(c, BAD_COL, v); continue; }
+            if (wt == 0) fail(c, BAD_WEIGHT, v);
+            if (u == v) fail(c, BAD_SELF, v);
+            if (e > row[v] && col[e - 1] >= u) fail(c, BAD_ORDER, v);
             gap += u > v ? u - v : v - u;
             wmax = max(wmax, wt);
             wmin = min(wmin, wt);
             wsum += wt;
-            fp += arc_hash(uint32_t(v), u, wt) - arc_hash(u, uint32_t(v), wt);
+            fp += arc_hash(v, u, wt) - arc_hash(u, v, wt);
         }
+        __syncwarp();
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -171,8 +238,24 @@ __global__ void check_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_
     }
     wmax = __reduce_max_sync(0xffffffffu, wmax);
     wmin = __reduce_min_sync(0xffffffffu, wmin);
-    if (lane == 0 && fp) atomicAdd(&c->fp, fp);
-    if (lane == 0 && wsum) {
+    if (lane == 0) {
+        part[0][warp] = fp;
+        part[1][warp] = gap;
+        part[2][warp] = wsum;
+        most[warp] = wmax;
+        least[warp] = wmin;
+    }
+    __syncthreads();
+    if (threadIdx.x) return;
+    for (int k = 1; k < ARC_TPB / 32; ++k) {
+        fp += part[0][k];
+        gap += part[1][k];
+        wsum += part[2][k];
+        wmax = max(wmax, most[k]);
+        wmin = min(wmin, least[k]);
+    }
+    if (fp) atomicAdd(&c->fp, fp);
+    if (wsum) {
         atomicAdd(&c->gap, gap);
         atomicAdd(&c->wsum, wsum);
         atomicMax(&c->wmax, wmax);
@@ -237,20 +320,44 @@ __global__ void rank_degree_kernel(uint32_t n, const uint64_t *row, const uint32
     }
 }
 
-// one warp per vertex: copy its row with neighbours renumbered (vert_at null: as
-// they are)
-__global__ void rank_arcs_kernel(uint32_t n, const uint64_t *row, const uint32_t *col,
-                                 const uint32_t *w, const uint32_t *vert_at,
-                                 const uint32_t *pos_of, const uint64_t *nrow, uint2 *arc) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warps = (uint64_t(gridDim.x) * blockDim.x) >> 5;
-    for (uint64_t p = (uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; p < n; p += warps) {
-        const uint32_t v = vert_at ? vert_at[p] : uint32_t(p);
-        const uint64_t a = row[v], b = row[v + 1], o = nrow[p];
-        for (uint64_t e = a + lane; e < b; e += 32) {
-            arc[o + (e - a)] = make_uint2(vert_at ? pos_of[col[e]] : col[e], w[e]);
+// the arcs in rank order, neighbours renumbered: arc i of the new order belongs
+// to the vertex of the position whose new row holds i
+__global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
+    rank_arcs_kernel(uint32_t n, uint64_t m2, uint64_t per_warp, const uint64_t *row, const uint32_t *col,
+                     const uint32_t *w, const uint32_t *vert_at, const uint32_t *pos_of, const uint64_t *nrow,
+                     uint2 *arc) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t lo = (uint64_t(blockIdx.x) * (ARC_TPB / 32) + (threadIdx.x >> 5)) * per_warp;
+    const uint64_t hi = min(lo + per_warp, m2);
+    uint32_t row0 = lo < hi ? row_of(n, nrow, lo) : 0;
+    for (uint64_t e0 = lo; e0 < hi; e0 += ARC_STEP) {
+        uint64_t src[ARC_STEP / 32];
+#pragma unroll
+        for (int k = 0; k < ARC_STEP / 32; ++k) {
+            const uint64_t b = e0 + 32 * k;
+            if (b >= hi) break;
+            const uint32_t last = uint32_t(min(hi - b, uint64_t(32))) - 1;
+            const uint32_t p = rows_of_step(n, nrow, b, last, row0);
+            src[k] = row[vert_at[p]] + (b + min(lane, last) - nrow[p]);
         }
+        uint32_t u[ARC_STEP / 32], wt[ARC_STEP / 32];
+#pragma unroll
+        for (int k = 0; k < ARC_STEP / 32; ++k)
+            if (e0 + 32 * k + lane < hi) {
+                u[k] = col[src[k]];
+                wt[k] = w[src[k]];
+            }
+#pragma unroll
+        for (int k = 0; k < ARC_STEP / 32; ++k)
+            if (e0 + 32 * k + lane < hi) arc[e0 + 32 * k + lane] = make_uint2(pos_of[u[k]], wt[k]);
+        __syncwarp();
     }
+}
+
+// the arcs as they are (the caller's numbering kept)
+__global__ void pack_arcs_kernel(uint64_t m2, const uint32_t *col, const uint32_t *w, uint2 *arc) {
+    for (uint64_t e = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < m2; e += uint64_t(gridDim.x) * blockDim.x)
+        arc[e] = make_uint2(col[e], w[e]);
 }
 
 int grid_for(uint64_t work, int tpb) {
@@ -289,6 +396,12 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     Check hchk{};
     uint32_t *cnt = nullptr;
     uint64_t *deg = nullptr;
+    // an equal piece of the arcs for each warp, in whole steps
+    const uint64_t arc_steps = (m2 + ARC_STEP - 1) / ARC_STEP;
+    const uint64_t arc_warps = std::min<uint64_t>(std::max<uint64_t>(arc_steps, 1),
+                                                  uint64_t(device_sms()) * ARC_BLOCKS * (ARC_TPB / 32));
+    const uint64_t per_warp = std::max<uint64_t>((arc_steps + arc_warps - 1) / arc_warps, 1) * ARC_STEP;
+    const unsigned arc_blocks = unsigned((arc_warps + ARC_TPB / 32 - 1) / (ARC_TPB / 32));
     g = RankGraph{};
     g.n = n;
     g.m2 = m2;
@@ -302,7 +415,7 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     check_rows_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, m2, row, chk);
     rank_count_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, rank, cnt, chk);
     rank_perm_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, rank, cnt, g.pos_of, g.vert_at, chk);
-    check_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, chk);
+    check_arcs_kernel<<<arc_blocks, ARC_TPB, 0, s>>>(n, m2, per_warp, row, col, w, chk);
     *launches += 4;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&hchk, chk, sizeof(Check), cudaMemcpyDeviceToHost, s));
@@ -355,8 +468,11 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
         CK(cudaMemsetAsync(deg + n, 0, sizeof(uint64_t), s));
         CK(exclusive_scan_u64(deg, g.row, uint64_t(n) + 1, s, launches));
     }
-    rank_arcs_kernel<<<grid_for(uint64_t(n) * 32, 256), 256, 0, s>>>(n, row, col, w, g.caller_ids ? nullptr : g.vert_at,
-                                                                     g.pos_of, g.row, g.arc);
+    if (g.caller_ids)
+        pack_arcs_kernel<<<grid_for(m2, 256), 256, 0, s>>>(m2, col, w, g.arc);
+    else
+        rank_arcs_kernel<<<arc_blocks, ARC_TPB, 0, s>>>(n, m2, per_warp, row, col, w, g.vert_at, g.pos_of, g.row,
+                                                       g.arc);
     *launches += 1;
     CK(cudaGetLastError());
     g.w_max = m2 ? hchk.wmax : 1;
