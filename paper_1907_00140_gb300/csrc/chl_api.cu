@@ -1827,6 +1827,15 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
     Params bestP{};
     float best_ms = -1.0f;
     unsigned long long best_stats[4] = {0, 0, 0, 0};
+    // Windows whose lists outgrow STATE_BYTES are no candidates: the trials time
+    // the trees alone, and such a build maps gigabytes anew each time (a
+    // 262,000-vertex grid at 256 threads and 64 buckets, 86 GB of lists: 193 ms,
+    // of which 141 in the trees).
+    auto lists_too_big = [&](const chl_build_opts &q) {
+        size_t fb = 0, tb = 0;
+        cudaMemGetInfo(&fb, &tb);
+        return double(choose_params(rg, q, sms, fb).list_words()) * 4.0 * double(n) > STATE_BYTES;
+    };
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (g->mem == CHL_MEM_HOST) {
@@ -1891,7 +1900,7 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
         else tpts = {256, 128, 512, 1024};
         std::vector<int> wins;
         if (o.window_buckets) wins.push_back(o.window_buckets);
-        else wins = {32, 16, 64};
+        else wins = {0, 16, 64};  // (0: what a build takes by default)
         auto run = [&](uint32_t d, int t, int w, Params *outP, float *outms,
                        unsigned long long *st4) -> chl_status {
             chl_build_opts q = o;
@@ -1923,11 +1932,15 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
             if (ms >= 0 && (best_ms < 0 || ms < best_ms)) { best_ms = ms; bestP = P; std::copy(st4, st4 + 4, best_stats); }
         }
         for (size_t i = 1; i < tpts.size(); ++i) {
-            st = run(bestP.delta, tpts[i], int(bestP.nwin), &P, &ms, st4);
+            st = run(bestP.delta, tpts[i], wins[0], &P, &ms, st4);
             if (st != CHL_OK) goto done;
             if (ms >= 0 && ms < best_ms) { best_ms = ms; bestP = P; std::copy(st4, st4 + 4, best_stats); }
         }
         for (size_t i = 1; i < wins.size(); ++i) {
+            chl_build_opts q = o;
+            q.threads_per_tree = bestP.tpt;
+            q.window_buckets = wins[i];
+            if (wins[i] == int(bestP.nwin) || lists_too_big(q)) continue;
             st = run(bestP.delta, bestP.tpt, wins[i], &P, &ms, st4);
             if (st != CHL_OK) goto done;
             if (ms >= 0 && ms < best_ms) { best_ms = ms; bestP = P; std::copy(st4, st4 + 4, best_stats); }
@@ -1962,15 +1975,20 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
             return CHL_OK;
         };
         if (!o.threads_per_tree) {
-            int best_tpt = bestP.tpt;
-            for (int t : {256, 512, 1024}) {
+            int best_tpt = bestP.tpt, best_win = best->window_buckets;
+            std::vector<int> ts = {256, 512, 1024};
+            if (rg.deg_max <= DIRECT_DEGREE) ts.push_back(128);
+            for (int t : ts) {
                 chl_build_opts q = *best;
                 q.threads_per_tree = t;
+                // (more slots may leave room for fewer lists each)
+                if (!o.window_buckets && q.window_buckets > 16 && lists_too_big(q)) q.window_buckets = 16;
                 double ms = 0;
                 if ((st = whole(q, &ms)) != CHL_OK) goto done;
-                if (best_build < 0 || ms < best_build) { best_build = ms; best_tpt = t; }
+                if (best_build < 0 || ms < best_build) { best_build = ms; best_tpt = t; best_win = q.window_buckets; }
             }
             best->threads_per_tree = best_tpt;
+            best->window_buckets = best_win;
         } else {
             if ((st = whole(*best, &best_build)) != CHL_OK) goto done;
         }
