@@ -57,17 +57,16 @@ WORKLOAD_TEXT = {
 }
 QUERIES = {"ba2k": 100_000}  # per-step query batch of each workload (default: --queries)
 
-# DRAM read + write bytes of plant_trees_kernel over one whole build (the sum
-# of dram__bytes_read.sum + dram__bytes_write.sum over its launches, one ncu
+# DRAM read + write bytes of the tree kernels over one whole build (the sum
+# of dram__bytes_read.sum + dram__bytes_write.sum over their launches, one ncu
 # capture of the current kernel source), keyed by workload, threads per tree,
 # bucket width, whether the build ran label-pruned phases, the big-tree
 # bucket width setting and the Common Label Table's size; other builds report
 # no traffic
 TREE_DRAM_BYTES_PER_BUILD = {
     # captured with overlap_phases=-1 (ncu serialises the second stream)
-    ("rmat18", 1024, 1, True, 0, 0): 31.955e9 + 8.734e9,
-    ("rmat18", 1024, 1, True, 0, 4): 29.428e9 + 8.107e9,
-    ("rmat18", 1024, 2, True, 0, 4): 29.785e9 + 8.236e9,
+    ("rmat18", 1024, 1, True, 0, 0): 23.518e9 + 7.757e9,
+    ("rmat18", 1024, 2, True, 0, 0): 23.723e9 + 7.791e9,
 }
 
 
@@ -314,7 +313,7 @@ def roofline(name, stats, tree_ms, opts, peak, peak_kind):
     traffic = TREE_DRAM_BYTES_PER_BUILD.get(key)
     return {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
             "traffic": traffic,
-            "traffic_note": ("DRAM read + write bytes of the tree kernel over one whole build "
+            "traffic_note": ("DRAM read + write bytes of the tree kernels over one whole build "
                              "(all its launches), from one ncu capture of the same build and "
                              "launch parameters; per build, like achieved" if traffic else
                              "null: no ncu capture of this workload and these launch parameters "

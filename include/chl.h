@@ -102,7 +102,9 @@ typedef struct chl_labels chl_labels;
  *                          Trees are independent (Sec. 5.2), so disjoint
  *                          ranges partition the labels by hub.
  *   threads_per_tree       CUDA threads cooperating on one tree (a power of
- *                          two in [32, 1024])
+ *                          two in [32, 1024]); 0 = by size: 1024, fewer for
+ *                          graphs of up to 131,072 arcs and for graphs whose
+ *                          rows all have at most 8 arcs
  *   bucket_delta           distance width of one bucket of the tree search
  *                          (>= 1)
  *   window_buckets         buckets held in the near window (2..64)
@@ -121,7 +123,12 @@ typedef struct chl_labels chl_labels;
  *                          skips (no label, no relaxation) a vertex whose
  *                          distance query on that table is at most its tree
  *                          distance. The labels are unchanged. 0 = the paper's
- *                          eta = 16; negative = no table; at most
+ *                          eta = 16, of which the phases that prune with the
+ *                          labels of earlier phases look at the top 4 (those
+ *                          labels hold the others too), and later phases leave
+ *                          the table out once it prunes under 1% of a phase's
+ *                          expansions; a value set here holds for every phase;
+ *                          negative = no table; at most
  *                          CHL_MAX_COMMON_HUBS. Requested trees of the eta
  *                          most important roots are built unpruned.
  *   pruned_bucket_delta    bucket width of the hybrid phases that prune with
@@ -164,7 +171,10 @@ typedef struct chl_labels chl_labels;
  *                          this, the later phases (whose trees are smaller
  *                          still) run small_threads_per_tree threads per tree,
  *                          so that more trees share each SM and hide each
- *                          other's per-tree latency. 0 = 8192
+ *                          other's per-tree latency. 0 = 8192. (Phases of
+ *                          16,384 roots and more whose trees expand at most a
+ *                          few hundred vertices hold whole trees in shared
+ *                          memory, whatever is set here.)
  *   small_threads_per_tree threads per tree after that switch (a power of two
  *                          in [32, 1024]); 0 = 256 (or pruned_threads_per_tree
  *                          when smaller)
@@ -172,9 +182,11 @@ typedef struct chl_labels chl_labels;
  *                          phase's trees averaged at least 45% of the vertices
  *                          (big trees: narrow buckets cut the re-expansions of
  *                          a label-correcting search by more than they add in
- *                          rounds); 0 = pruned_bucket_delta / 16 (at least 1),
+ *                          rounds); 0 = pruned_bucket_delta / 16 (at least 1)
+ *                          for graphs of 131,072 vertices and more,
  *                          negative = pruned_bucket_delta for every phase
- *   overlap_phases         0 = on: while a label-pruned phase's last trees run,
+ *   overlap_phases         0 = on (for graphs of 32,768 vertices and more, where
+ *                          it pays): while a label-pruned phase's last trees run,
  *                          the SMs they leave idle start the next phase's
  *                          first trees on a second stream, pruned by the
  *                          current (older) table; the labels are the same.
@@ -307,7 +319,8 @@ chl_status chl_build(const chl_csr *g, const uint32_t *rank, const chl_build_opt
  * sample has the build's mix of large and small trees) for candidate bucket
  * widths, then block sizes, then window sizes (coordinate search), and the
  * fastest is kept. For a whole build (no root range set in base) the block
- * size is then settled by whole builds (256, 512 and 1024 threads), since the
+ * size is then settled by whole builds (256, 512 and 1024 threads, and 128
+ * where every row has at most 8 arcs), since the
  * hybrid phases prune later trees far below the sample's sizes, and then the
  * phases' switch points, each by whole builds: the first-phase switch
  * (switch_ratio default or off), the frontier size of the small-tree switch

@@ -26,7 +26,7 @@
 // builds it; so the class of table (threads, slots) is only a matter of speed.
 //
 // Bound by instruction issue of the few warps that the tables leave room for
-// (10 CTAs of 64 threads per SM; a quarter of the issue slots, 1.5 of 15 cycles
+// (9 or 12 CTAs of 64 threads per SM; a quarter of the issue slots, 1.5 of 15 cycles
 // per instruction on global loads), where the general kernel waits on global
 // memory. So it wins where trees are tiny and many: R-MAT scale 18 roots
 // [38912, 155648) 0.79 -> 0.35 ms, [9728, 38912) 1.70 -> 1.32 ms, a 50,000-vertex
