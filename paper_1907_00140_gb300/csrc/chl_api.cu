@@ -94,18 +94,21 @@ namespace {
 // Host-mapped staging of the query calls: the kernel sets its bad-vertex flag
 // in it, and a batch of up to STAGE_PAIRS host pairs is read from it and
 // answered into it, so that such a call is one launch and one wait (an
-// allocation, a memset and up to three copies before: one pair 44 us, now 21).
+// allocation, a memset and up to three copies before: one pair 53 us, now 25 to 26).
 // A call takes a block and gives it back before it returns, so blocks are never
-// shared between threads or streams; at most STAGE_BLOCKS exist, of which
-// STAGE_IDLE stay allocated while no call uses them. A call that gets none
-// takes the general path. The pairs are copied into the block before the stream
-// gets to them: earlier work on the stream may still write them, so the call
-// compares them again after its wait, and where they differ it is made anew
-// with copies on the stream (asking the stream first cost 4 to 7 us a call).
+// shared between threads or streams. The STAGE_BLOCKS blocks (393 KB) are one
+// allocation, made by the first call and kept: page-locked memory is slow to
+// allocate and to free, and freeing it waits for the work of every stream, so
+// a short query beside a long build would wait for the build. A call that finds
+// every block taken goes the general path. The pairs are copied into the block
+// before the stream gets to them: earlier work on the stream may still write
+// them, so the call compares them again after its wait, and where they differ it
+// is made anew with copies on the stream (asking the stream first cost 4 to 7 us
+// a call).
 constexpr uint64_t STAGE_PAIRS = 4096;
-constexpr int STAGE_BLOCKS = 8, STAGE_IDLE = 2;
+constexpr int STAGE_BLOCKS = 8;
 
-struct StageBlock {
+struct alignas(128) StageBlock {
     uint32_t pairs[2 * STAGE_PAIRS];
     uint32_t out[STAGE_PAIRS];
     int bad;
@@ -114,43 +117,37 @@ struct StageBlock {
 struct Stage {
     StageBlock *b = nullptr;
     static std::mutex mu;
-    static StageBlock *idle[STAGE_IDLE];
-    static int n_idle, made;
+    static StageBlock *idle[STAGE_BLOCKS];
+    static int n_idle;
+    static bool made;
     Stage() {
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            if (n_idle) b = idle[--n_idle];
-            else if (made < STAGE_BLOCKS) ++made;
-            else return;
-        }
-        if (!b) {
-            void *p = nullptr;
-            if (cudaHostAlloc(&p, sizeof(StageBlock), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
-                b = static_cast<StageBlock *>(p);
-            } else {
-                (void)cudaGetLastError();
-                std::lock_guard<std::mutex> lk(mu);
-                --made;
-                return;
-            }
-        }
+        std::lock_guard<std::mutex> lk(mu);
+        if (!made) make();
+        if (!n_idle) return;
+        b = idle[--n_idle];
         b->bad = 0;
     }
     ~Stage() {
         if (!b) return;
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            if (n_idle < STAGE_IDLE) {
-                idle[n_idle++] = b;
-                return;
-            }
-            --made;
-        }
-        cudaFreeHost(b);
+        std::lock_guard<std::mutex> lk(mu);
+        idle[n_idle++] = b;
     }
     Stage(const Stage &) = delete;
     Stage &operator=(const Stage &) = delete;
+
+private:
+    static void make() {  // (under mu)
+        void *p = nullptr;
+        if (cudaHostAlloc(&p, STAGE_BLOCKS * sizeof(StageBlock), cudaHostAllocPortable | cudaHostAllocMapped) !=
+            cudaSuccess) {
+            (void)cudaGetLastError();  // the general path, and another try by the next call
+            return;
+        }
+        for (; n_idle < STAGE_BLOCKS; ++n_idle) idle[n_idle] = static_cast<StageBlock *>(p) + n_idle;
+        made = true;
+    }
 };
+
 // host memory that the host itself may copy from and to (not managed, not a
 // device address)
 bool plain_host(const void *p) {
@@ -163,8 +160,9 @@ bool plain_host(const void *p) {
 }
 
 std::mutex Stage::mu;
-StageBlock *Stage::idle[STAGE_IDLE] = {};
-int Stage::n_idle = 0, Stage::made = 0;
+StageBlock *Stage::idle[STAGE_BLOCKS] = {};
+int Stage::n_idle = 0;
+bool Stage::made = false;
 
 // device control block of one tree launch; the two counters every tree
 // updates sit on cache lines of their own
