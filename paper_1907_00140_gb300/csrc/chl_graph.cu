@@ -155,11 +155,16 @@ __device__ __forceinline__ uint32_t row_of(uint32_t n, const uint64_t *row, uint
 
 // The row of arc e0 + min(lane, last) on each lane of a warp. v: a row at or
 // before that of e0, with no whole row of arcs between; on return the row of the
-// last of these arcs. 32 row ends a turn, looked up by shuffles.
+// last of these arcs. 32 row ends a turn, looked up by shuffles; a run of
+// EMPTY_TURNS turns over rows without arcs ends in a search for the row of the
+// next arc, so that no warp walks a long run of isolated vertices alone (10^7 of
+// them between the arcs: a build 390 ms, now 200, as with them at the end).
+constexpr int EMPTY_TURNS = 8;
 __device__ __forceinline__ uint32_t rows_of_step(uint32_t n, const uint64_t *row, uint64_t e0, uint32_t last,
                                                  uint32_t &v) {
     const uint32_t lane = threadIdx.x & 31, at = min(lane, last);
-    uint32_t r = 0;
+    uint32_t r = 0, next = 0;  // arcs before `next` have their row
+    int empty = 0;
     bool found = false;
     for (;;) {
         const uint64_t i = uint64_t(v) + 1 + lane;
@@ -176,6 +181,12 @@ __device__ __forceinline__ uint32_t rows_of_step(uint32_t n, const uint64_t *row
         }
         if (top > last) break;
         v += 32;
+        empty = top == next ? empty + 1 : 0;
+        next = top;
+        if (empty == EMPTY_TURNS) {
+            v = row_of(n, row, e0 + next);
+            empty = 0;
+        }
     }
     v = __shfl_sync(0xffffffffu, r, 31);
     return r;
