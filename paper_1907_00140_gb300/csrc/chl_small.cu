@@ -72,7 +72,7 @@ struct Tree {
     uint32_t n_out, n_put;
     uint32_t max_d;           // largest label distance (all trees)
     unsigned long long base;
-    unsigned long long n_exp[TPB / 32], n_arcs[TPB / 32], n_pruned[TPB / 32];  // statistics per warp
+    unsigned long long n_exp[TPB / 32], n_arcs[TPB / 32], n_pruned[TPB / 32];  // statistics of this tree per warp
     // label-pruned phases only (the launch leaves the rest out otherwise)
     uint32_t lth_key[LTH_SLOTS], lth_val[LTH_SLOTS];
     uint32_t lth_bit[ROOT_BITS / 32];  // by hub position modulo ROOT_BITS
@@ -195,8 +195,9 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         S.key[i] = key_inf<K>();
     }
     if (tid == 0) S.max_d = 0;
-    if (lane == 0) S.n_exp[tid >> 5] = S.n_arcs[tid >> 5] = S.n_pruned[tid >> 5] = 0;
-    unsigned long long n_rounds = 0, n_buckets = 0, n_trees = 0;
+    // launch statistics, of the trees built here: a spilled tree's work is counted
+    // by the kernel that builds it (the first three on lane 0, of its warp)
+    unsigned long long n_exp = 0, n_arcs = 0, n_pruned = 0, n_rounds = 0, n_buckets = 0, n_trees = 0;
 
     for (;;) {
         __syncthreads();  // the previous tree's table is clean, S.root is read
@@ -217,6 +218,8 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         const uint32_t h = S.root;
         if (h == NONE) break;
         const uint32_t hv = root_vertex<K>(p, h);
+        uint32_t rounds = 0, buckets = 0;
+        if (lane == 0) S.n_exp[tid >> 5] = S.n_arcs[tid >> 5] = S.n_pruned[tid >> 5] = 0;
         // the pruning tables of the root (see chl_tree.cu)
         const bool prune = p.hc && h >= p.hc_hubs;
         if (prune)
@@ -257,7 +260,6 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
             uint32_t n_pend = 1, b = 0;
             int x = 0, r = 0;
             bool entered = true;  // the current bucket was entered by this round
-            uint32_t rounds = 0;
             for (;;) {
                 // ---- scan the pending vertices
                 Counters &c = S.c[r];
@@ -354,7 +356,6 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                     }
                     __syncthreads();
                 }
-                ++n_rounds;
                 if (S.over || S.stop) break;
                 if (++rounds > p.round_limit) {
                     if (tid == 0) atomicExch(&p.flags[0], ERR_ROUND_LIMIT);
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
                 n_pend = c.n_next;
                 if (!n_pend) break;
                 entered = c.minb > b;
-                n_buckets += entered;
+                buckets += entered;
                 b = c.minb;
                 x ^= 1;
                 r ^= 1;
@@ -382,6 +383,13 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
             continue;
         }
         ++n_trees;
+        n_rounds += rounds;
+        n_buckets += buckets;
+        if (lane == 0) {
+            n_exp += S.n_exp[tid >> 5];
+            n_arcs += S.n_arcs[tid >> 5];
+            n_pruned += S.n_pruned[tid >> 5];
+        }
         // ---- emission: count, reserve the tree's output range, write, reset
         const uint32_t nt = S.n_touch;
         uint32_t mine = 0, far = 0;
@@ -441,9 +449,9 @@ __global__ void __launch_bounds__(TPB) plant_small_kernel(TreeLaunch p, uint32_t
         }
     }
     if (lane == 0) {
-        if (S.n_exp[tid >> 5]) atomicAdd(&p.stats[0], S.n_exp[tid >> 5]);
-        if (S.n_arcs[tid >> 5]) atomicAdd(&p.stats[1], S.n_arcs[tid >> 5]);
-        if (S.n_pruned[tid >> 5]) atomicAdd(&p.stats[6], S.n_pruned[tid >> 5]);
+        if (n_exp) atomicAdd(&p.stats[0], n_exp);
+        if (n_arcs) atomicAdd(&p.stats[1], n_arcs);
+        if (n_pruned) atomicAdd(&p.stats[6], n_pruned);
     }
     if (tid == 0) {
         atomicAdd(&p.stats[3], n_trees);

@@ -1,8 +1,8 @@
 """Trees built in shared memory (phases of many tiny trees) and rows relaxed by
 one thread (graphs of degree at most 8), against the oracle: every key layout,
-trees that outgrow the table (spilled to the general kernel), roots with more
-table labels than their hash holds, and a label buffer that fills up while
-spilled roots wait. Integers: comparisons are exact."""
+trees that outgrow the table (spilled to the general kernel, and counted once),
+roots with more table labels than their hash holds, and a label buffer that
+fills up while spilled roots wait. Integers: comparisons are exact."""
 import re
 
 import numpy as np
@@ -75,6 +75,22 @@ def test_small_trees_equal_oracle(built, opts, capfd, monkeypatch):
         for v in (1, 700, 1499):  # the parent on a line ranked from its start is the vertex before
             a, b = int(off[v]), int(off[v + 1])
             assert np.array_equal(par[a:b], np.where(hub[a:b] == v, v, v - 1))
+
+
+def test_spilled_trees_are_counted_once(capfd, monkeypatch):
+    """On paths every vertex of a tree is expanded once, so without label pruning
+    (and with one table throughout) the statistics do not depend on the kernel."""
+    g, rank = case("line")
+    monkeypatch.setenv("CHL_TRACE", "1")
+    fixed = dict(switch_ratio=-1.0, psi_threshold=1e9, common_hubs=16)
+    got = []
+    for opts in (fixed, dict(fixed, small_threads_per_tree=256)):
+        capfd.readouterr()
+        st = chl.build_labels(DG(g), dev(rank), **opts).stats()
+        seen = [(int(c), int(s)) for c, s in re.findall(r"class (-?\d+) spilled (\d+)", capfd.readouterr().err)]
+        got.append(({k: st[k] for k in ("trees", "trivial", "labels", "expanded", "arcs", "pruned")}, seen))
+    assert any(c >= 0 and s > 100 for c, s in got[0][1]) and all(c < 0 for c, _ in got[1][1]), got
+    assert got[0][0] == got[1][0]
 
 
 @pytest.mark.parametrize("tpt", [32, 64, 128, 256, 512, 1024])
