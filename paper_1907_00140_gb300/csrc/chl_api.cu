@@ -1153,13 +1153,16 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
                 }
             }
             pending = failed;
-            if (first && tiny >= 0 && hc.spill_n > hc.next_spill) {
-                // spilled roots that no launch claimed
-                const size_t k = hc.spill_n - hc.next_spill;
-                pending.resize(failed.size() + k);
-                CUDA_TRY(cudaMemcpy(pending.data() + failed.size(), (const uint32_t *)b_spill.p + hc.next_spill, k * 4,
-                                    cudaMemcpyDeviceToHost));
+            // spilled roots that no launch claimed
+            const size_t left = first && tiny >= 0 && hc.spill_n > hc.next_spill ? hc.spill_n - hc.next_spill : 0;
+            if (left) {
+                pending.resize(failed.size() + left);
+                CUDA_TRY(cudaMemcpy(pending.data() + failed.size(), (const uint32_t *)b_spill.p + hc.next_spill,
+                                    left * 4, cudaMemcpyDeviceToHost));
             }
+            if (trace)
+                std::fprintf(stderr, "chl phase %zu label buffer full: %zu roots did not fit, %zu spilled ones wait\n",
+                             ph, failed.size(), left);
             for (uint32_t i = claimed_upto; i < count; ++i) pending.push_back(root_at(i));
             first = false;
             if (attempt > 40) {

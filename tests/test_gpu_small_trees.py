@@ -77,6 +77,26 @@ def test_small_trees_equal_oracle(built, opts, capfd, monkeypatch):
             assert np.array_equal(par[a:b], np.where(hub[a:b] == v, v, v - 1))
 
 
+def test_full_buffer_while_spilled_roots_wait(capfd, monkeypatch):
+    """The label buffer fills up in the shared-memory launch of a phase: the roots
+    spilled by then are claimed by no launch and built after the buffer has grown."""
+    g, rank = case("line")
+    ref = O.build_labels(g, rank, "plant", threads=8)
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    chl.build_labels(DG(g), dev(rank)).free()
+    phases = [[int(x) for x in m] for m in re.findall(
+        r"roots \[(\d+), (\d+)\).* class (-?\d+) spilled (\d+) .* labels (\d+) rounds", capfd.readouterr().err)]
+    k = max((i for i, p in enumerate(phases) if p[2] >= 0), key=lambda i: phases[i][3])
+    assert phases[k][3] > 100, phases
+    # room for the phase's trivial roots and for few of the others
+    room = sum(p[4] for p in phases[:k]) + phases[k][1] - phases[k][0]
+    L = chl.build_labels(DG(g), dev(rank), label_capacity=room)
+    waited = [int(x) for x in re.findall(r"(\d+) spilled ones wait", capfd.readouterr().err)]
+    assert any(waited), (waited, phases)
+    assert_same(ref, *L.to_numpy())
+
+
 def test_spilled_trees_are_counted_once(capfd, monkeypatch):
     """On paths every vertex of a tree is expanded once, so without label pruning
     (and with one table throughout) the statistics do not depend on the kernel."""
