@@ -182,8 +182,9 @@ typedef struct chl_labels chl_labels;
  *                          phase's trees averaged at least 45% of the vertices
  *                          (big trees: narrow buckets cut the re-expansions of
  *                          a label-correcting search by more than they add in
- *                          rounds); 0 = pruned_bucket_delta / 16 (at least 1)
- *                          for graphs of 131,072 vertices and more,
+ *                          rounds); 0 = pruned_bucket_delta / 16 (at least 1),
+ *                          in graphs of fewer than 131,072 vertices only after
+ *                          a phase that was label-pruned itself;
  *                          negative = pruned_bucket_delta for every phase
  *   overlap_phases         0 = on (for graphs of 32,768 vertices and more, where
  *                          it pays): while a label-pruned phase's last trees run,

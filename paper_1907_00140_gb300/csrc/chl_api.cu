@@ -228,8 +228,14 @@ constexpr double STATE_BYTES = 24.0 * (1 << 30);
 // 0.51 ms there, 0.83 ms here).
 constexpr double SMALL_EXPANSIONS[SMALL_CLASSES] = {96, 300, 600};
 constexpr uint32_t SMALL_ROOTS = 16384;
-// ... of at least this many vertices (77,000: 10.46 ms with it, 10.27 without;
-// 174,000: 41.0 and 41.4; 1.24 million: 698 and 767)
+// The narrow width after big trees, by default, in graphs of at least this many
+// vertices (77,000: 10.46 ms with it, 10.27 without; 174,000: 41.0 and 41.4; 1.24
+// million: 698 and 767); in smaller ones only where label pruning has left the
+// trees big: scale-free trees shrink in the first label-pruned phase (R-MAT scale
+// 16 6.8 ms with the width in that phase, 6.6 without, 50,000-vertex BA 9.3 and
+// 8.8), those of random graphs stay big for several phases (20,000 vertices of
+// degree 40 123 ms with it, 154 without, of degree 80 177 and 247; 40,000 of
+// degree 40 697 and 994).
 constexpr uint32_t BIG_TREE_N = 131072;
 // graphs below this many vertices run their phases one after the other: the
 // second stream's launches cost more than the tails they fill (24,000 vertices:
@@ -323,7 +329,6 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     p.delta_lt = o.pruned_bucket_delta > 0 ? uint32_t(o.pruned_bucket_delta) : dl;
     p.delta_big = o.big_tree_bucket_delta > 0   ? uint32_t(o.big_tree_bucket_delta)
                   : o.big_tree_bucket_delta < 0 ? 0u
-                        : g.n < BIG_TREE_N      ? 0u
                                                 : std::max<uint32_t>(1u, p.delta_lt / 16);
     p.nwin = o.window_buckets > 0 ? uint32_t(o.window_buckets) : 32;
     // 4-byte keys hold distances up to 2^31 - 2; every tentative distance of a
@@ -1214,7 +1219,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     // when this phase's averaged BIG_TREE_COVER of the vertices
     {
         const uint64_t built = (agg[3] - tr0) - (agg[2] - triv0);
-        big = built && double(agg[0] - exp0) / double(built) >= BIG_TREE_COVER * double(n);
+        big = built && double(agg[0] - exp0) / double(built) >= BIG_TREE_COVER * double(n) &&
+              (ph_lt || n >= BIG_TREE_N || o.big_tree_bucket_delta > 0);
     }
     const uint32_t table_hubs = use_lt && !o.common_hubs ? std::min(P.eta, LT_COMMON_HUBS) : P.eta;
     if (hybrid && (!table.buf.p || (table.hubs != table_hubs && !lt.offsets))) {

@@ -24,6 +24,7 @@ if not torch.cuda.is_available():
 import paper_1907_00140_gb300 as chl  # noqa: E402
 
 from test_gpu_parity import DG, dev, assert_same  # noqa: E402
+from test_gpu_query_blocks import graph_of  # noqa: E402
 
 NEVER_SMALL = 1               # no tree averages fewer than one expansion
 ALWAYS_SMALL = 0xFFFFFFFF     # every label-pruned phase's trees average fewer
@@ -121,3 +122,25 @@ def test_tuned_switch_points_are_exact(family):
     got = L.query(dev(pairs)).cpu().numpy().view(np.uint32)
     assert np.array_equal(got, O.query(ref, rank, pairs, threads=8))
     L.free()
+
+
+@pytest.mark.parametrize("kind,first,later", [("random", False, True), ("scale-free", False, False)])
+def test_narrow_width_after_big_pruned_trees(kind, first, later, capfd, monkeypatch):
+    """Small graphs take the narrow width where a label-pruned phase's trees were
+    still big (random graphs), not after the unpruned first phase."""
+    rng = np.random.default_rng(2)
+    if kind == "random":
+        a, b = rng.integers(0, 4000, (2, 80_000))
+        on = a != b
+        key = np.unique(np.minimum(a, b)[on] * 4000 + np.maximum(a, b)[on])
+        g = graph_of(4000, key // 4000, key % 4000, rng.integers(1, 101, len(key)))
+        rank = W.degree_rank(g)
+    else:
+        g, rank = W.load("ba2k")
+    ref = O.build_labels(g, rank, "plant", threads=8)
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    L = chl.build_labels(DG(g), dev(rank), switch_ratio=1e6, small_tree_expansions=NEVER_SMALL)
+    narrow = [" narrow" in x for x in capfd.readouterr().err.splitlines() if "table 1" in x]
+    assert narrow[0] == first and any(narrow[1:]) == later, narrow
+    assert_same(ref, *L.to_numpy())
