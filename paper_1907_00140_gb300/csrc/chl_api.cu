@@ -1166,8 +1166,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
                                     left * 4, cudaMemcpyDeviceToHost));
             }
             if (trace)
-                std::fprintf(stderr, "chl phase %zu label buffer full: %zu roots did not fit, %zu spilled ones wait\n",
-                             ph, failed.size(), left);
+                std::fprintf(stderr, "chl phase %zu label buffer full: %zu roots did not fit (%zu overlapped ones did not "
+                             "fit theirs), %zu spilled ones wait\n", ph, failed.size(), ffailed.size(), left);
             for (uint32_t i = claimed_upto; i < count; ++i) pending.push_back(root_at(i));
             first = false;
             if (attempt > 40) {

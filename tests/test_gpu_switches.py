@@ -9,6 +9,8 @@ of work changes: the label table of earlier phases covers a rank-closed hub
 set whenever it is used (Sec. 5.3), and the small-tree launch runs the same
 search in smaller blocks. Each build's statistics show which switch fired.
 """
+import re
+
 import numpy as np
 import pytest
 
@@ -143,4 +145,51 @@ def test_narrow_width_after_big_pruned_trees(kind, first, later, capfd, monkeypa
     L = chl.build_labels(DG(g), dev(rank), switch_ratio=1e6, small_tree_expansions=NEVER_SMALL)
     narrow = [" narrow" in x for x in capfd.readouterr().err.splitlines() if "table 1" in x]
     assert narrow[0] == first and any(narrow[1:]) == later, narrow
+    assert_same(ref, *L.to_numpy())
+
+
+def line_before_scale_free(n, line, wave):
+    """Pairs of vertices at the first 2 * wave positions, among them (in the second
+    wave) the head of a long path; then a scale-free graph of n vertices; the rest
+    of the path last. The path's tree is the long tail of the second phase, and the
+    next phase's first trees label nearly n vertices each."""
+    rng = np.random.default_rng(8)
+    ba = W.barabasi_albert(n, 5, seed=8, wlo=1, whi=100)
+    u, v, w = ba.edges()
+    pairs = 2 * np.arange(wave)
+    at = n + 2 * wave
+    head = n + wave + wave // 2
+    path = np.concatenate([[head], at + np.arange(line)])
+    a = np.concatenate([u, n + pairs, path[:-1]]).astype(np.int64)
+    b = np.concatenate([v, n + pairs + 1, path[1:]]).astype(np.int64)
+    g = graph_of(at + line, a, b, np.concatenate([w, rng.integers(1, 100, wave + line)]).astype(np.int64))
+    pos = np.empty(g.n, np.int64)
+    pos[n:at] = np.arange(2 * wave)
+    pos[:n] = 2 * wave + (n - 1 - W.degree_rank(ba).astype(np.int64))
+    pos[at:] = at + np.arange(line)
+    return g, (g.n - 1 - pos).astype(np.uint32)
+
+
+@pytest.fixture(scope="module")
+def long_tail():
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g, rank = line_before_scale_free(33_000, 3000, sms)
+    return g, rank, O.build_labels(g, rank, "plant", threads=8)
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(flags=chl.CHL_FLAG_PARENTS), dict(label_capacity=1000)],
+                         ids=["default", "parents", "full buffer"])
+def test_overlapped_trees(long_tail, opts, capfd, monkeypatch):
+    """The next phase's first trees in a phase's tail, on a graph large enough for
+    them by default; with a small label buffer they overflow theirs and are built
+    again by their own phase."""
+    g, rank, ref = long_tail
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    L = chl.build_labels(DG(g), dev(rank), switch_ratio=1e6, **opts)
+    err = capfd.readouterr().err
+    if "label_capacity" in opts:
+        assert any(int(x) for x in re.findall(r"(\d+) overlapped ones did not fit", err)), err
+    else:
+        assert L.stats()["overlapped_trees"] > 0, err
     assert_same(ref, *L.to_numpy())
