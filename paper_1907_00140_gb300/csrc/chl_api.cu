@@ -318,7 +318,15 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     // 1, 7.25 at 4 and 8, 8.0 at 16, and with weights to 100,000, 7.9 at 512, 7.7 at
     // 1024, 8.5 at 2048; scale 17 with weights to 1000, 18.4 at 1, 14.1 at 8, 16.2
     // at 32; scale 18, 41.0 at 1, 40.3 at 2; scale 21, 690 at 4 and at 8).
-    const double dflt = mean_deg >= 8.0 ? std::max(g.w_mean / 64.0, 1400.0 * g.w_mean / double(g.n))
+    // Heavy-tailed weights take narrower buckets: wide ones expand vertices long
+    // before their distances are known, and the Common Label Table prunes those, so
+    // that the switch to label pruning fires too early (random graph of 60,000
+    // vertices, degree 16, weights log-uniform to 100,000: 1,114 ms at width 256, 611
+    // at 64, R-MAT scale 16 12.8 and 14.9 ms; one edge in a hundred of weight
+    // 100,000: 739 and 652 ms, R-MAT 10.4 and 10.2).
+    const double dflt = mean_deg >= 8.0 ? (g.w_spread > HEAVY_SPREAD
+                                               ? g.w_mean / 128.0
+                                               : std::max(g.w_mean / 64.0, 1400.0 * g.w_mean / double(g.n)))
                         : p.direct && g.w_min * 4.0 >= g.w_mean ? double(g.w_min) : 2.0 * g.w_mean;
     uint32_t d = 1;  // default: the power of two nearest to dflt
     while (double(d) * 1.5 < dflt && d < (1u << 30)) d <<= 1;
@@ -852,6 +860,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     const int ph_tiny = tiny;
     const bool ph_narrow = big && P.delta_big && lt.offsets;
     const int ph_lt = lt.offsets ? 1 : 0;
+    const uint32_t ph_width = ph_narrow ? P.delta_big : ph_lt ? P.delta_lt : P.delta;
     if (trace) t_ph = now_ms();
     if (lt.offsets) ++lt_phases;
     if (small) ++small_phases;
@@ -1284,9 +1293,9 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     if (trace) {
         CUDA_TRY(cudaStreamSynchronize(s));
         std::fprintf(stderr,
-                     "chl phase %zu roots [%u, %u) table %d%s%s class %d spilled %u trees %.3f ms assemble %.3f ms "
+                     "chl phase %zu roots [%u, %u) table %d%s%s width %u class %d spilled %u trees %.3f ms assemble %.3f ms "
                      "expanded %llu arcs %llu labels %llu rounds %llu buckets %llu pruned %llu\n",
-                     ph, pb, pe, ph_lt, ph_small ? " small" : "", ph_narrow ? " narrow" : "", ph_tiny, hc.spill_n, t_tree,
+                     ph, pb, pe, ph_lt, ph_small ? " small" : "", ph_narrow ? " narrow" : "", ph_width, ph_tiny, hc.spill_n, t_tree,
                      now_ms() - t_ph - t_tree,
                      (unsigned long long)(agg[0] - exp0), (unsigned long long)(agg[1] - arc0),
                      (unsigned long long)(T - T0), (unsigned long long)(agg[4] - rd0),

@@ -102,6 +102,7 @@ struct Check {
     uint32_t deg_max;  // longest row
     uint32_t wmax, wmin;
     unsigned long long wsum;
+    double wsq;             // sum of the squared weights
     unsigned long long gap; // sum of |u - v| over the arcs
     unsigned long long fp;  // symmetry fingerprint: sum of h(v, u, w) - h(u, v, w) over the arcs
 };
@@ -207,9 +208,11 @@ __global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
                       const uint32_t *w, Check *c) {
     if (*(volatile uint32_t *)&c->bits & (BAD_ROWPTR | BAD_RANK)) return;
     __shared__ unsigned long long part[3][ARC_TPB / 32];
+    __shared__ float part_sq[ARC_TPB / 32];
     __shared__ uint32_t most[ARC_TPB / 32], least[ARC_TPB / 32];
     uint32_t wmax = 0, wmin = 0xFFFFFFFFu;
     unsigned long long wsum = 0;
+    float wsq = 0.0f;  // (for a launch rule: rounding does not matter)
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long fp = 0, gap = 0;
     const uint64_t lo = (uint64_t(blockIdx.x) * (ARC_TPB / 32) + warp) * per_warp, hi = min(lo + per_warp, m2);
@@ -237,6 +240,7 @@ __global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
             wmax = max(wmax, wt);
             wmin = min(wmin, wt);
             wsum += wt;
+            wsq += float(wt) * float(wt);
             fp += arc_hash(v, u, wt) - arc_hash(u, v, wt);
         }
         __syncwarp();
@@ -246,6 +250,7 @@ __global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
         fp += __shfl_xor_sync(0xffffffffu, fp, o);
         gap += __shfl_xor_sync(0xffffffffu, gap, o);
         wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+        wsq += __shfl_xor_sync(0xffffffffu, wsq, o);
     }
     wmax = __reduce_max_sync(0xffffffffu, wmax);
     wmin = __reduce_min_sync(0xffffffffu, wmin);
@@ -253,6 +258,7 @@ __global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
         part[0][warp] = fp;
         part[1][warp] = gap;
         part[2][warp] = wsum;
+        part_sq[warp] = wsq;
         most[warp] = wmax;
         least[warp] = wmin;
     }
@@ -262,6 +268,7 @@ __global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
         fp += part[0][k];
         gap += part[1][k];
         wsum += part[2][k];
+        wsq += part_sq[k];
         wmax = max(wmax, most[k]);
         wmin = min(wmin, least[k]);
     }
@@ -269,6 +276,7 @@ __global__ void __launch_bounds__(ARC_TPB, ARC_BLOCKS)
     if (wsum) {
         atomicAdd(&c->gap, gap);
         atomicAdd(&c->wsum, wsum);
+        atomicAdd(&c->wsq, double(wsq));
         atomicMax(&c->wmax, wmax);
         atomicMin(&c->wmin, wmin);
     }
@@ -489,6 +497,7 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     g.w_max = m2 ? hchk.wmax : 1;
     g.w_min = m2 ? hchk.wmin : 1;
     g.w_mean = m2 ? double(hchk.wsum) / double(m2) : 1.0;
+    g.w_spread = m2 ? hchk.wsq / double(m2) / (g.w_mean * g.w_mean) : 1.0;
 done:
     if (chk) cudaFreeAsync(chk, s);
     if (cnt) cudaFreeAsync(cnt, s);

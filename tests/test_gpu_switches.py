@@ -148,6 +148,34 @@ def test_narrow_width_after_big_pruned_trees(kind, first, later, capfd, monkeypa
     assert_same(ref, *L.to_numpy())
 
 
+@pytest.mark.parametrize("kind", ["uniform", "log-uniform", "few heavy", "huge"])
+def test_bucket_width_by_spread_of_the_weights(kind, capfd, monkeypatch):
+    """The default width of an unpruned phase: from the mean weight and the vertex
+    count, narrower for heavy-tailed weights (mean square above four squared means)."""
+    rng = np.random.default_rng(3)
+    n, m = 3000, 30_000
+    u, v = rng.integers(0, n, (2, m))
+    on = u != v
+    key = np.unique(np.minimum(u, v)[on] * n + np.maximum(u, v)[on])
+    m = len(key)
+    w = {"uniform": rng.integers(1, 101, m), "log-uniform": np.exp(rng.random(m) * np.log(100_000)).astype(np.int64) + 1,
+         "few heavy": np.where(rng.random(m) < 0.01, 100_000, rng.integers(1, 11, m)),
+         "huge": np.where(rng.random(m) < 0.001, 2**30, rng.integers(1, 11, m))}[kind]
+    g = graph_of(n, key // n, key % n, w)
+    rank = W.degree_rank(g)
+    mean, square = float(w.mean()), float((w.astype(np.float64) ** 2).mean())
+    want = mean / 128 if square > 4 * mean * mean else max(mean / 64, 1400 * mean / n)
+    assert (square > 4 * mean * mean) == (kind != "uniform")
+    width = 1
+    while width * 1.5 < want:
+        width *= 2
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    L = chl.build_labels(DG(g), dev(rank))
+    assert int(re.search(r" width (\d+) ", capfd.readouterr().err).group(1)) == width
+    assert_same(O.build_labels(g, rank, "plant", threads=8), *L.to_numpy())
+
+
 def line_before_scale_free(n, line, wave):
     """Pairs of vertices at the first 2 * wave positions, among them (in the second
     wave) the head of a long path; then a scale-free graph of n vertices; the rest
