@@ -252,8 +252,20 @@ constexpr uint32_t LT_COMMON_HUBS = 4;
 constexpr uint32_t ROOT_ARRAY_BYTES = 64u << 10;
 
 // vertices up to which a graph with short rows runs 128 instead of 256 threads
-// per tree
+// per tree (grids of 131,000 to 202,000: 128 threads faster by 0 to 2%; 262,000:
+// 126 ms at 256 threads, 136 at 128)
 constexpr uint32_t DIRECT_SMALL_N = 131072;
+// Graphs with short rows whose trees stay narrow (grids expand 60 to 130 vertices
+// a round) want those block sizes, graphs whose trees do not want 1024 threads:
+// builds at 128 and 1024 threads, random 6-regular, 60,000 vertices (2,500 a
+// round) 822 and 371 ms, random cubic, 30,000 (570) 59 and 52, 3-d mesh, 64,000
+// (390) 199 and 175, 140,000 (470) 599 and 864, randomly numbered grid, 90,000
+// (90) 51 and 111. Local numberings are narrow enough (at most 2% slower than at 1024
+// threads before), and up to DIRECT_SURE_N vertices 128 threads won on every graph
+// tried; the others begin at 1024 threads and leave them where the first trees
+// expand fewer than WIDE_ROUND vertices a round.
+constexpr uint32_t DIRECT_SURE_N = 20000;
+constexpr double WIDE_ROUND = 512.0;
 
 struct Params {
     int tpt;
@@ -278,6 +290,7 @@ struct Params {
     uint32_t fin_words;  // settled-filter bitmap words per CTA
     uint32_t w_min;
     int direct;  // short rows only (TreeLaunch::direct)
+    bool unsure; // ... of trees that may be wide (see WIDE_ROUND)
     uint32_t n;
     int max_slots() const { return std::max(slots, std::max(slots_lt, slots_sm)); }
     // list words per vertex over all slots, the largest of the launches' layouts
@@ -303,8 +316,14 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     // Small graphs leave most of 1024 threads idle too (at 256 / 512 / 1024: 11,900
     // arcs 0.95 / 1.04 / 1.06, 120,000 arcs 2.78 / 2.54 / 2.81, 190,000 arcs 2.43 /
     // 1.99 / 1.74).
+    // Heavy-tailed weights want wide buckets in few trees at once: the first
+    // phase's trees, which no labels prune, are one per slot (grid with log-uniform
+    // weights, 25,600 vertices: 98 ms at 128 threads, of which 91 in that phase's
+    // 1,368 trees; 30 at 1024 threads).
+    const bool narrow = p.direct && g.w_spread <= HEAVY_SPREAD;
+    p.unsure = narrow && !o.threads_per_tree && !g.local && g.n > DIRECT_SURE_N;
     p.tpt = o.threads_per_tree ? o.threads_per_tree
-            : p.direct         ? (g.n <= DIRECT_SMALL_N ? 128 : 256)
+            : narrow           ? (g.n <= DIRECT_SMALL_N ? 128 : 256)
             : g.m2 <= 16384    ? 256
             : g.m2 <= 131072   ? 512
                                : 1024;
@@ -409,6 +428,21 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     p.slots = int(slots);
     p.slots_lt = int(slots_lt);
     return p;
+}
+
+// P with 1024 threads per tree: fewer of its slots, of the same layout
+void widen(Params &P, const chl_build_opts &o, int sms) {
+    auto at_most = [&](int slots, uint32_t fin_words, uint32_t aux) {
+        return o.slots > 0 ? slots : std::min(slots, sms * std::max(plant_max_slots_per_sm(1024, fin_words, aux), 1));
+    };
+    uint32_t aux = 0;
+    P.tpt = 1024;
+    plant_smem_split(1024, P.n, 0, &P.fin_words, &aux);
+    P.slots = at_most(P.slots, P.fin_words, 0);
+    if (o.pruned_threads_per_tree) return;
+    P.tpt_lt = 1024;
+    plant_smem_split(1024, P.n, P.stage_want ? P.stage_want : ROOT_ARRAY_BYTES, &P.fin_words_lt, &P.aux_lt);
+    P.slots_lt = at_most(P.slots_lt, P.fin_words_lt, P.aux_lt);
 }
 
 // The class of the shared-memory tree kernel for a phase of `roots` roots whose
@@ -707,7 +741,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     SlotState slot;
     CommonTable table;
     RankGraph rg;
-    Params P{};
+    Params P{}, P_narrow{};
+    bool undecided = false;  // P is P_narrow widened until trees have shown their width
     Control hc{};
     Control *ctl = nullptr;
     LabelCSR csr;
@@ -803,6 +838,11 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     }
 
     CUDA_TRY(slot.alloc(P, n, s));
+    if (o.mode == 0 && P.unsure) {
+        P_narrow = P;
+        undecided = true;
+        widen(P, o, sms);
+    }
     CUDA_TRY(dmalloc(&b_ctl.p, sizeof(Control), s));
     ctl = (Control *)b_ctl.p;
     CUDA_TRY(dmalloc(&b_fail.p, size_t(re - rb + 1) * 4, s));
@@ -841,9 +881,12 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     // the Common Label Table is needed when some requested tree lies outside
     // it; a hybrid build takes it from its first phase instead
     if (P.eta && re > P.eta && !hybrid) {
-        st = build_common_table(rg, P, slot, s, table, &launches, nullptr);
+        unsigned long long seen[7] = {};
+        st = build_common_table(rg, P, slot, s, table, &launches, seen);
         if (st != CHL_OK) goto done;
         with_table = true;
+        if (undecided && double(seen[0]) < WIDE_ROUND * double(seen[4])) P = P_narrow;
+        undecided = false;
     }
     CUDA_TRY(cudaEventRecord(ev[4], s));
     phases.clear();
@@ -859,6 +902,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     const bool ph_small = small;
     const int ph_tiny = tiny;
     const bool ph_narrow = big && P.delta_big && lt.offsets;
+    const int ph_threads = lt.offsets ? (small ? P.tpt_sm : P.tpt_lt) : P.tpt;
     const int ph_lt = lt.offsets ? 1 : 0;
     const uint32_t ph_width = ph_narrow ? P.delta_big : ph_lt ? P.delta_lt : P.delta;
     if (trace) t_ph = now_ms();
@@ -1192,6 +1236,8 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
             cap *= 2;
         }
     }
+    if (undecided && double(agg[0] - exp0) < WIDE_ROUND * double(agg[4] - rd0)) P = P_narrow;
+    undecided = false;
     // The switch of Sec. 5.2: label pruning starts once a phase's trees explore
     // many vertices per label (Psi = expansions / labels above psi_th), or once
     // the Common Label Table pruned a large share of their expansions; before
@@ -1293,9 +1339,9 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     if (trace) {
         CUDA_TRY(cudaStreamSynchronize(s));
         std::fprintf(stderr,
-                     "chl phase %zu roots [%u, %u) table %d%s%s width %u class %d spilled %u trees %.3f ms assemble %.3f ms "
+                     "chl phase %zu roots [%u, %u) table %d%s%s threads %d width %u class %d spilled %u trees %.3f ms assemble %.3f ms "
                      "expanded %llu arcs %llu labels %llu rounds %llu buckets %llu pruned %llu\n",
-                     ph, pb, pe, ph_lt, ph_small ? " small" : "", ph_narrow ? " narrow" : "", ph_width, ph_tiny, hc.spill_n, t_tree,
+                     ph, pb, pe, ph_lt, ph_small ? " small" : "", ph_narrow ? " narrow" : "", ph_threads, ph_width, ph_tiny, hc.spill_n, t_tree,
                      now_ms() - t_ph - t_tree,
                      (unsigned long long)(agg[0] - exp0), (unsigned long long)(agg[1] - arc0),
                      (unsigned long long)(T - T0), (unsigned long long)(agg[4] - rd0),

@@ -37,6 +37,7 @@ struct RankGraph {
     uint32_t *pos_of = nullptr;  // [n] caller vertex id -> pos
     uint32_t w_max = 0, w_min = 0;
     uint32_t deg_max = 0;        // longest row
+    bool local = false;          // neighbours lie close together in the caller's numbering
     bool caller_ids = false;     // vertices numbered as by the caller
     const uint32_t *vertex_pos() const { return caller_ids ? pos_of : nullptr; }
     // index of a caller's vertex in this graph: null = as it is

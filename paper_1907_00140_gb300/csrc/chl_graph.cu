@@ -404,7 +404,9 @@ int grid_for(uint64_t work, int tpb) {
 // vertices: 143 ms by rank, 127 ms so; 90,000: 33.5 and 32.1; 49,000 and fewer:
 // within 1%, the rank order stays). Scale-free graphs gain more from the rank
 // order, which puts the hubs together.
-static constexpr double LOCAL_GAP = 1.0 / 16;
+// Light-tailed weights only: the block sizes of the other graphs with short rows
+// (choose_params) have no kernels for the caller's numbering.
+static constexpr double LOCAL_GAP = 1.0 / 128;
 static constexpr uint32_t LOCAL_N = 65536;
 
 chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uint32_t *col,
@@ -478,7 +480,10 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(dmalloc(&g.row, (size_t(n) + 1) * sizeof(uint64_t), s));
     CK(dmalloc(&g.arc, (m2 ? m2 : 1) * sizeof(uint2), s));
     g.deg_max = hchk.deg_max;
-    g.caller_ids = keep_ids && n >= LOCAL_N && m2 && g.deg_max <= DIRECT_DEGREE && double(hchk.gap) / double(m2) < double(n) * LOCAL_GAP;
+    g.w_mean = m2 ? double(hchk.wsum) / double(m2) : 1.0;
+    g.w_spread = m2 ? hchk.wsq / double(m2) / (g.w_mean * g.w_mean) : 1.0;
+    g.local = m2 && double(hchk.gap) / double(m2) < double(n) * LOCAL_GAP;
+    g.caller_ids = keep_ids && n >= LOCAL_N && g.local && g.deg_max <= DIRECT_DEGREE && g.w_spread <= HEAVY_SPREAD;
     if (g.caller_ids) {
         CK(cudaMemcpyAsync(g.row, row, (size_t(n) + 1) * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
     } else {
@@ -496,8 +501,6 @@ chl_status prepare_graph(uint32_t n, uint64_t m2, const uint64_t *row, const uin
     CK(cudaGetLastError());
     g.w_max = m2 ? hchk.wmax : 1;
     g.w_min = m2 ? hchk.wmin : 1;
-    g.w_mean = m2 ? double(hchk.wsum) / double(m2) : 1.0;
-    g.w_spread = m2 ? hchk.wsq / double(m2) / (g.w_mean * g.w_mean) : 1.0;
 done:
     if (chk) cudaFreeAsync(chk, s);
     if (cnt) cudaFreeAsync(cnt, s);

@@ -132,3 +132,51 @@ def test_short_rows_every_block_size(tpt, flags):
     ref = O.build_labels(g, rank, "plant", threads=8)
     L = chl.build_labels(DG(g), dev(rank), threads_per_tree=tpt, flags=flags)
     assert_same(ref, *L.to_numpy())
+
+
+def short_rows(name):
+    rng = np.random.default_rng(17)
+    if name == "tree":  # wide trees: a complete binary tree in heap order, ranked by depth
+        n = 2**18 - 1
+        i = np.arange(1, n)
+        return graph_of(n, (i - 1) // 2, i, rng.integers(1, 50, n - 1)), np.arange(n - 1, -1, -1).astype(np.uint32)
+    g = W.grid(100 if name == "small mixed grid" else 150, 100, seed=5)
+    u, v, w = (x.astype(np.int64) for x in g.edges())
+    if name == "heavy grid":
+        w = np.exp(rng.random(len(w)) * np.log(100_000)).astype(np.int64) + 1
+    new = np.arange(g.n) if name in ("grid", "heavy grid") else rng.permutation(g.n)
+    rank = np.empty(g.n, np.uint32)
+    rank[new] = W.spt_count_rank(g, 16, seed=5)
+    return graph_of(g.n, new[u], new[v], w), rank
+
+
+# threads per tree in the first phase, in the later ones, in a build of a root range with and without a table
+@pytest.mark.parametrize("name,first,later,ranged,bare", [
+    ("grid", 128, 128, 128, 128), ("small mixed grid", 128, 128, 128, 128), ("mixed grid", 1024, 128, 128, 1024),
+    ("tree", 1024, 1024, 1024, 1024), ("heavy grid", 512, 512, 512, 512)])
+def test_block_size_of_short_rows(name, first, later, ranged, bare, capfd, monkeypatch):
+    """Local numberings and small graphs take few threads per tree, other graphs
+    once their first trees have shown that they are narrow, heavy-tailed weights the
+    general rule."""
+    g, rank = short_rows(name)
+    ref = O.build_labels(g, rank, "plant", threads=8)
+    d, r = DG(g), dev(rank)
+    monkeypatch.setenv("CHL_TRACE", "1")
+
+    def threads(**opts):
+        capfd.readouterr()
+        L = chl.build_labels(d, r, small_tree_expansions=1, **opts)
+        return L, [int(x) for x in re.findall(r" threads (\d+) ", capfd.readouterr().err)]
+
+    L, seen = threads()
+    assert len(seen) > 1 and seen[0] == first and set(seen[1:]) == {later}, seen
+    assert_same(ref, *L.to_numpy())
+    for opts, want in ((dict(), ranged), (dict(common_hubs=-1), bare)):
+        L, seen = threads(root_begin=100, root_end=2000, **opts)
+        assert seen == [want], (seen, opts)
+        off, hub, dist = L.to_numpy()
+        pos = g.n - 1 - rank.astype(np.int64)
+        v = np.repeat(np.arange(g.n), np.diff(ref.offsets.astype(np.int64)))
+        on = (pos[ref.hub] >= 100) & (pos[ref.hub] < 2000)
+        assert np.array_equal(hub, ref.hub[on]) and np.array_equal(dist, ref.dist[on])
+        assert np.array_equal(np.diff(off.astype(np.int64)), np.bincount(v[on], minlength=g.n))
