@@ -180,3 +180,28 @@ def test_block_size_of_short_rows(name, first, later, ranged, bare, capfd, monke
         on = (pos[ref.hub] >= 100) & (pos[ref.hub] < 2000)
         assert np.array_equal(hub, ref.hub[on]) and np.array_equal(dist, ref.dist[on])
         assert np.array_equal(np.diff(off.astype(np.int64)), np.bincount(v[on], minlength=g.n))
+
+
+def test_label_buffer_of_large_road_like_graphs(capfd, monkeypatch):
+    """Four grids of 420 x 420 side by side (about 390 labels per vertex): the label
+    buffer holds them at once, so that no tree is built twice; the labels are those
+    of one grid."""
+    g = W.grid(420, 35_000, seed=42)
+    u, v, w = (x.astype(np.int64) for x in g.edges())
+    rank = W.spt_count_rank(g, 16, seed=42).astype(np.int64)
+    one = chl.build_labels(DG(g), dev(rank.astype(np.uint32)))
+    k = np.repeat(np.arange(4), len(u)) * g.n
+    four = graph_of(4 * g.n, np.tile(u, 4) + k, np.tile(v, 4) + k, np.tile(w, 4))
+    assert four.n * 512 * 12 > 4 << 30
+    rank4 = (4 * np.tile(rank, 4) + np.repeat(np.arange(4), g.n)).astype(np.uint32)
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    L = chl.build_labels(DG(four), dev(rank4))
+    assert "label buffer full" not in capfd.readouterr().err
+    st = L.stats()
+    assert st["trees"] == four.n and st["labels"] == 4 * one.total > 256 * four.n
+    off, hub, dist = one.to_numpy()
+    off4, hub4, dist4 = L.to_numpy()
+    for i in (0, 3):
+        a, b = int(off4[i * g.n]), int(off4[(i + 1) * g.n])
+        assert np.array_equal(hub4[a:b] - np.uint32(i * g.n), hub) and np.array_equal(dist4[a:b], dist)
