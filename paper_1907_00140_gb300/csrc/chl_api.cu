@@ -430,6 +430,12 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     return p;
 }
 
+// block sizes given by the caller may have no kernel for its numbering
+bool may_keep_ids(const chl_build_opts &o) {
+    auto fits = [](int threads) { return !threads || caller_ids_block(threads); };
+    return o.mode == 0 && fits(o.threads_per_tree) && fits(o.pruned_threads_per_tree) && fits(o.small_threads_per_tree);
+}
+
 // P with 1024 threads per tree: fewer of its slots, of the same layout
 void widen(Params &P, const chl_build_opts &o, int sms) {
     auto at_most = [&](int slots, uint32_t fin_words, uint32_t aux) {
@@ -771,10 +777,6 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     uint64_t lt_records = 0;  // output records the label table holds
     unsigned long long max_dist = 0;  // largest label distance so far
     const double psi_th = o.psi_threshold > 0.0f ? double(o.psi_threshold) : PSI_TH;
-    // block sizes given by the caller may have no kernel for its numbering
-    const bool keep_ids = o.mode == 0 && (!o.threads_per_tree || caller_ids_block(o.threads_per_tree)) &&
-                          (!o.pruned_threads_per_tree || caller_ids_block(o.pruned_threads_per_tree)) &&
-                          (!o.small_threads_per_tree || caller_ids_block(o.small_threads_per_tree));
     uint32_t claimed_upto = 0;
     bool first = true;
     Filler fill[2];                  // next-phase trees in a phase's tail, by phase parity
@@ -815,7 +817,7 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
         d_w = (const uint32_t *)b_w.p;
         d_rank = (const uint32_t *)b_rank.p;
     }
-    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, keep_ids, rg, s, &launches);
+    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, may_keep_ids(o), rg, s, &launches);
     if (st != CHL_OK) goto done;
 
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
@@ -1918,8 +1920,10 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
         d_w = (const uint32_t *)b_w.p;
         d_rank = (const uint32_t *)b_rank.p;
     }
-    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, false, rg, s, &launches);
+    st = prepare_graph(n, m2, d_row, d_col, d_w, d_rank, may_keep_ids(o), rg, s, &launches);
     if (st != CHL_OK) goto done;
+    if (std::getenv("CHL_TRACE") && std::getenv("CHL_TRACE")[0] == '1')
+        std::fprintf(stderr, "chl tune trials in %s\n", rg.caller_ids ? "the caller's numbering" : "rank order");
     CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     {
         // rank-strided sample: every (n/K)-th rank position, about four trees per slot
@@ -1961,6 +1965,7 @@ extern "C" chl_status chl_tune(const chl_csr *g, const uint32_t *rank, const chl
         }
         std::vector<int> tpts;
         if (o.threads_per_tree) tpts.push_back(o.threads_per_tree);
+        else if (rg.caller_ids) tpts = {256, 128};  // as the builds of these block sizes; the others are tried by whole builds
         else tpts = {256, 128, 512, 1024};
         std::vector<int> wins;
         if (o.window_buckets) wins.push_back(o.window_buckets);

@@ -205,3 +205,18 @@ def test_label_buffer_of_large_road_like_graphs(capfd, monkeypatch):
     for i in (0, 3):
         a, b = int(off4[i * g.n]), int(off4[(i + 1) * g.n])
         assert np.array_equal(hub4[a:b] - np.uint32(i * g.n), hub) and np.array_equal(dist4[a:b], dist)
+
+
+@pytest.mark.parametrize("fixed,numbering", [(dict(), "the caller's numbering"),
+                                             (dict(threads_per_tree=512), "rank order")])
+def test_tuning_trials_run_the_kernels_of_the_build(fixed, numbering, capfd, monkeypatch):
+    """A graph that a build keeps in the caller's numbering is tuned in it."""
+    g, rank = case("grid280")
+    d, r = DG(g), dev(rank)
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    opts, rep = chl.tune(d, r, **fixed)
+    assert re.findall(r"chl tune trials in (.*)", capfd.readouterr().err) == [numbering]
+    want, got = chl.build_labels(d, r), chl.build_labels(d, r, **opts)
+    for x, y in zip(want.to_numpy(), got.to_numpy()):
+        assert np.array_equal(x, y)
