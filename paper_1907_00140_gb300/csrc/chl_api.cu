@@ -1699,7 +1699,7 @@ extern "C" chl_status chl_path(const chl_labels *L, const uint32_t *pairs, uint6
         dpath = (uint32_t *)b_path.p;
         dlen = (uint32_t *)b_len.p;
     }
-    CUDA_TRY(launch_paths(L->n, L->offsets, L->hubpos, L->dist, L->hub, L->parent, dp, q, max_len,
+    CUDA_TRY(launch_paths(L->n, L->offsets, L->hubpos, L->dist, L->parent, dp, q, max_len,
                           dpath, dlen, bad, s));
     if (mem == CHL_MEM_HOST) {
         if (max_len) CUDA_TRY(cudaMemcpyAsync(paths, dpath, q * max_len * 4, cudaMemcpyDeviceToHost, s));

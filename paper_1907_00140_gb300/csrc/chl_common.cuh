@@ -220,8 +220,8 @@ cudaError_t launch_query(uint32_t n, const uint64_t *offsets, const uint32_t *hu
 // shortest paths from parents stored with the labels; bad = 1 for an id >= n,
 // 2 for a broken parent chain
 cudaError_t launch_paths(uint32_t n, const uint64_t *offsets, const uint32_t *hubpos,
-                         const uint32_t *dist, const uint32_t *hub, const uint32_t *parent,
-                         const uint32_t *pairs, uint64_t q, uint32_t max_len, uint32_t *paths,
+                         const uint32_t *dist, const uint32_t *parent, const uint32_t *pairs,
+                         uint64_t q, uint32_t max_len, uint32_t *paths,
                          uint32_t *lens, int *bad, cudaStream_t s);
 // one resident label set as the query kernels read it: its lists, or (nparts
 // > 0) its hub partitions, a device array of nparts sets over the same n
@@ -239,7 +239,7 @@ struct QuerySet {
 // which the pairs are answered (launch_group_order)
 cudaError_t launch_query_sets(const QuerySet *sets, const uint32_t *nsets, const uint32_t *pairs,
                               const uint16_t *set_of, const uint32_t *perm, uint64_t q, uint32_t *out,
-                              int *bad, int max_blocks, cudaStream_t s);
+                              int *bad, cudaStream_t s);
 // the same answers for one set given as a kernel parameter: its lists, or its
 // hub partitions (the minimum over them); perm as above
 struct QueryLists {
@@ -254,8 +254,7 @@ struct QueryParts {
 cudaError_t launch_query_parts(const QueryParts &sets, const uint32_t *pairs, const uint32_t *perm, uint64_t q,
                                uint32_t *out, int *bad, cudaStream_t s);
 // grouped order of a batch: perm[0..q) = the pairs sorted by the block pair of
-// their two vertices (64 blocks per set); set_of may be null (all set 0);
-// scratch holds 4096 counters
+// their two vertices (64 blocks per set); scratch holds 4096 counters
 constexpr uint32_t GROUP_SCRATCH_WORDS = 4096;
 cudaError_t launch_group_order(const QuerySet *sets, const uint32_t *nsets, const uint32_t *pairs,
                                const uint16_t *set_of, uint64_t q, uint32_t *scratch, uint32_t *perm,

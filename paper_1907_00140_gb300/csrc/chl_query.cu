@@ -302,8 +302,8 @@ constexpr int PATH_TPB = 128;
 
 __global__ void __launch_bounds__(PATH_TPB) paths_kernel(uint32_t n, const uint64_t *__restrict__ off,
                              const uint32_t *__restrict__ hp, const uint32_t *__restrict__ dd,
-                             const uint32_t *__restrict__ hub, const uint32_t *__restrict__ par,
-                             const uint32_t *__restrict__ pairs, uint64_t q, uint32_t max_len,
+                             const uint32_t *__restrict__ par, const uint32_t *__restrict__ pairs,
+                             uint64_t q, uint32_t max_len,
                              uint32_t *__restrict__ paths, uint32_t *__restrict__ lens, int *bad) {
     // the merge's table; between merges its space keeps the v side
     __shared__ __align__(16) uint32_t tabs[PATH_TPB / 32][TAB];
@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(QUERY_TPB, QUERY_CTAS) query_sets_kernel(const
         uint32_t k = 0xFFFFu, u = 0, v = 0, d = 0xFFFFFFFFu;
         if (mine) {
             i = perm ? __ldg(&perm[j]) : j;
-            k = set_of ? __ldg(&set_of[i]) : 0u;
+            k = __ldg(&set_of[i]);
             mine = k != 0xFFFFu;
         }
         bool ok = false;
@@ -492,7 +492,7 @@ struct GroupSets {
     __device__ __forceinline__ uint32_t key(const uint32_t *pairs, uint64_t i) const {
         uint32_t size = n;
         if (sets) {
-            const uint32_t k = set_of ? __ldg(&set_of[i]) : 0;
+            const uint32_t k = __ldg(&set_of[i]);
             if (k >= *nsets) return 0;
             size = sets[k].n;
         }
@@ -594,23 +594,21 @@ cudaError_t launch_query_parts(const QueryParts &sets, const uint32_t *pairs, co
 
 cudaError_t launch_query_sets(const QuerySet *sets, const uint32_t *nsets, const uint32_t *pairs,
                               const uint16_t *set_of, const uint32_t *perm, uint64_t q, uint32_t *out,
-                              int *bad, int max_blocks, cudaStream_t s) {
+                              int *bad, cudaStream_t s) {
     if (q == 0) return cudaSuccess;
-    uint64_t blocks = (q * 32 + 255) / 256;
-    if (blocks > uint64_t(max_blocks)) blocks = uint64_t(max_blocks);
-    blocks = resident_blocks(blocks);
+    const uint64_t blocks = resident_blocks((q * 32 + QUERY_TPB - 1) / QUERY_TPB);
     query_sets_kernel<<<unsigned(blocks), QUERY_TPB, 0, s>>>(sets, nsets, pairs, set_of, perm, q, out, bad);
     return cudaGetLastError();
 }
 
 cudaError_t launch_paths(uint32_t n, const uint64_t *offsets, const uint32_t *hubpos,
-                         const uint32_t *dist, const uint32_t *hub, const uint32_t *parent,
-                         const uint32_t *pairs, uint64_t q, uint32_t max_len, uint32_t *paths,
+                         const uint32_t *dist, const uint32_t *parent, const uint32_t *pairs,
+                         uint64_t q, uint32_t max_len, uint32_t *paths,
                          uint32_t *lens, int *bad, cudaStream_t s) {
     if (q == 0) return cudaSuccess;
     uint64_t blocks = (q * 32 + PATH_TPB - 1) / PATH_TPB;
     if (blocks > uint64_t(device_sms()) * 64) blocks = uint64_t(device_sms()) * 64;
-    paths_kernel<<<unsigned(blocks), PATH_TPB, 0, s>>>(n, offsets, hubpos, dist, hub, parent, pairs, q,
+    paths_kernel<<<unsigned(blocks), PATH_TPB, 0, s>>>(n, offsets, hubpos, dist, parent, pairs, q,
                                                    max_len, paths, lens, bad);
     return cudaGetLastError();
 }
@@ -619,8 +617,7 @@ cudaError_t launch_query(uint32_t n, const uint64_t *offsets, const uint32_t *hu
                          const uint32_t *dist, const uint32_t *pairs, uint64_t q, uint32_t *out,
                          int *bad, cudaStream_t s) {
     if (q == 0) return cudaSuccess;
-    uint64_t blocks = (q * 32 + 255) / 256;
-    blocks = resident_blocks(blocks);
+    const uint64_t blocks = resident_blocks((q * 32 + QUERY_TPB - 1) / QUERY_TPB);
     query_kernel<<<unsigned(blocks), QUERY_TPB, 0, s>>>(n, offsets, hubpos, dist, pairs, q, out, bad);
     return cudaGetLastError();
 }

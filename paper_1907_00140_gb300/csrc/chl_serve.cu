@@ -409,7 +409,7 @@ extern "C" chl_status chl_server_create(const chl_server_opts *opts, chl_server 
                 uint32_t *flag = sl.h_out + B;
                 launch_query_sets(S->d_sets, S->d_nsets, reinterpret_cast<const uint32_t *>(sl.h_in),
                                   reinterpret_cast<const uint16_t *>(sl.h_in + 8 * B), nullptr, B,
-                                  sl.h_out, reinterpret_cast<int *>(flag), S->sms * 64, sl.s);
+                                  sl.h_out, reinterpret_cast<int *>(flag), sl.s);
                 e = cudaStreamEndCapture(sl.s, &gph);
             } else if (!e) {
                 uint32_t *flag = sl.d_out + B;
@@ -422,7 +422,7 @@ extern "C" chl_status chl_server_create(const chl_server_opts *opts, chl_server 
                     launch_group_order(S->d_sets, S->d_nsets, pairs_d, set_d, B, sl.d_scratch, sl.d_perm, sl.s);
                 launch_query_sets(S->d_sets, S->d_nsets, pairs_d, set_d,
                                   o.query_order == 1 ? sl.d_perm : nullptr, B, sl.d_out,
-                                  reinterpret_cast<int *>(flag), S->sms * 64, sl.s);
+                                  reinterpret_cast<int *>(flag), sl.s);
                 cudaMemcpyAsync(sl.h_out, sl.d_out, B * 4 + 4, cudaMemcpyDeviceToHost, sl.s);
                 e = cudaStreamEndCapture(sl.s, &gph);
             }
