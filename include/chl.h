@@ -104,7 +104,9 @@ typedef struct chl_labels chl_labels;
  *   threads_per_tree       CUDA threads cooperating on one tree (a power of
  *                          two in [32, 1024]); 0 = by size: 1024, fewer for
  *                          graphs of up to 131,072 arcs and for graphs whose
- *                          rows all have at most 8 arcs
+ *                          rows all have at most 8 arcs and whose trees are
+ *                          narrow (small graphs and local numberings at once,
+ *                          others once their first trees have shown it)
  *   bucket_delta           distance width of one bucket of the tree search
  *                          (>= 1)
  *   window_buckets         buckets held in the near window (2..64)
@@ -183,8 +185,9 @@ typedef struct chl_labels chl_labels;
  *                          (big trees: narrow buckets cut the re-expansions of
  *                          a label-correcting search by more than they add in
  *                          rounds); 0 = pruned_bucket_delta / 16 (at least 1),
- *                          in graphs of fewer than 131,072 vertices only after
- *                          a phase that was label-pruned itself;
+ *                          in graphs of fewer than 131,072 vertices only from
+ *                          a label-pruned phase on whose trees averaged as many
+ *                          expansions as there are vertices;
  *                          negative = pruned_bucket_delta for every phase
  *   overlap_phases         0 = on (for graphs of 32,768 vertices and more, where
  *                          it pays): while a label-pruned phase's last trees run,

@@ -230,13 +230,15 @@ constexpr double SMALL_EXPANSIONS[SMALL_CLASSES] = {96, 300, 600};
 constexpr uint32_t SMALL_ROOTS = 16384;
 // The narrow width after big trees, by default, in graphs of at least this many
 // vertices (77,000: 10.46 ms with it, 10.27 without; 174,000: 41.0 and 41.4; 1.24
-// million: 698 and 767); in smaller ones only where label pruning has left the
-// trees big: scale-free trees shrink in the first label-pruned phase (R-MAT scale
-// 16 6.8 ms with the width in that phase, 6.6 without, 50,000-vertex BA 9.3 and
-// 8.8), those of random graphs stay big for several phases (20,000 vertices of
-// degree 40 123 ms with it, 154 without, of degree 80 177 and 247; 40,000 of
-// degree 40 697 and 994).
+// million: 698 and 767); in smaller ones only once a label-pruned phase's trees
+// expanded SMALL_TREE_COVER times the vertices, that is, the same ones again and
+// again: in scale-free graphs they average half the vertices (R-MAT scale 16
+// with the width in the first such phase 6.8 ms, in the next two 7.6 against 7.2,
+// without 6.6), in random graphs two to three times all of them for several phases
+// (20,000 vertices of degree 40 124 ms with it, 154 without, of degree 80 176 and
+// 247; 40,000 of degree 40 697 and 994).
 constexpr uint32_t BIG_TREE_N = 131072;
+constexpr double SMALL_TREE_COVER = 1.0;
 // graphs below this many vertices run their phases one after the other: the
 // second stream's launches cost more than the tails they fill (24,000 vertices:
 // 5.42 ms with them, 5.09 without; 50,000: 10.0 and 10.7)
@@ -315,7 +317,8 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
     // the last level cache).
     // Small graphs leave most of 1024 threads idle too (at 256 / 512 / 1024: 11,900
     // arcs 0.95 / 1.04 / 1.06, 120,000 arcs 2.78 / 2.54 / 2.81, 190,000 arcs 2.43 /
-    // 1.99 / 1.74).
+    // 1.99 / 1.74). The cuts are loose: Barabasi-Albert graphs of 18,000 arcs take
+    // 0.97 / 0.95 / 1.03, 36,000 1.49 / 1.39 / 1.36, 84,000 3.08 / 2.56 / 2.48.
     // Heavy-tailed weights want wide buckets in few trees at once: the first
     // phase's trees, which no labels prune, are one per slot (grid with log-uniform
     // weights, 25,600 vertices: 98 ms at 128 threads, of which 91 in that phase's
@@ -1278,8 +1281,9 @@ extern "C" chl_status chl_build(const chl_csr *g, const uint32_t *rank, const ch
     // when this phase's averaged BIG_TREE_COVER of the vertices
     {
         const uint64_t built = (agg[3] - tr0) - (agg[2] - triv0);
-        big = built && double(agg[0] - exp0) / double(built) >= BIG_TREE_COVER * double(n) &&
-              (ph_lt || n >= BIG_TREE_N || o.big_tree_bucket_delta > 0);
+        const bool large = n >= BIG_TREE_N || o.big_tree_bucket_delta > 0;
+        const double cover = large || ph_narrow ? BIG_TREE_COVER : SMALL_TREE_COVER;
+        big = built && (large || ph_lt) && double(agg[0] - exp0) / double(built) >= cover * double(n);
     }
     const uint32_t table_hubs = use_lt && !o.common_hubs ? std::min(P.eta, LT_COMMON_HUBS) : P.eta;
     if (hybrid && (!table.buf.p || (table.hubs != table_hubs && !lt.offsets))) {
