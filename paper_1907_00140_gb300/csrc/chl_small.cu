@@ -32,7 +32,8 @@
 // [38912, 155648) 0.79 -> 0.35 ms, [9728, 38912) 1.70 -> 1.32 ms, a 50,000-vertex
 // Barabasi-Albert graph's [9728, 38912) 1.94 -> 1.11 ms, the last 184,000 roots of
 // a 512x512 grid 15.6 -> 10.5 ms. Tables of 4,096 and 8,192 slots for trees of
-// about a thousand vertices lost to it by a factor of 1.4 to 2.5.
+// about a thousand vertices lost to it on that Barabasi-Albert graph (1.9 ms against
+// 4.3 and 5.8); they were not tried on grids.
 #include "chl_tree.cuh"
 
 namespace chl {

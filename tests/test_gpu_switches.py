@@ -128,8 +128,8 @@ def test_tuned_switch_points_are_exact(family):
 
 @pytest.mark.parametrize("kind,first,later", [("random", False, True), ("scale-free", False, False)])
 def test_narrow_width_after_big_pruned_trees(kind, first, later, capfd, monkeypatch):
-    """Small graphs take the narrow width where a label-pruned phase's trees were
-    still big (random graphs), not after the unpruned first phase."""
+    """Small graphs take the narrow width once a label-pruned phase's trees expanded
+    as many vertices as there are (random graphs), not after the unpruned first phase."""
     rng = np.random.default_rng(2)
     if kind == "random":
         a, b = rng.integers(0, 4000, (2, 80_000))
