@@ -330,6 +330,11 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
             : g.m2 <= 16384    ? 256
             : g.m2 <= 131072   ? 512
                                : 1024;
+    // Few threads suit many trees in flight. Where the caller limits them, a tree gets
+    // the threads that the limit leaves idle (270 x 270 grid at 16 / 64 / 304 / 608
+    // trees: 1,352 / 196 / 52 / 35 ms at 128 threads, 918 / 154 / 40 / 26 so).
+    if (narrow && !o.threads_per_tree && o.slots > 0)
+        while (p.tpt < 1024 && (long long)p.tpt * 2 * o.slots <= 1024ll * sms) p.tpt *= 2;
     const double mean_deg = g.n ? double(g.m2) / double(g.n) : 0.0;
     // ... and where no weight lies far below the mean, buckets as wide as the
     // lightest arc settle in one or two rounds instead of four (262,000-vertex
@@ -436,6 +441,8 @@ Params choose_params(const RankGraph &g, const chl_build_opts &o, int sms, size_
 // block sizes given by the caller may have no kernel for its numbering
 bool may_keep_ids(const chl_build_opts &o) {
     auto fits = [](int threads) { return !threads || caller_ids_block(threads); };
+    // (the limit that choose_params turns into 512 threads)
+    if (!o.threads_per_tree && o.slots > 0 && 512ll * o.slots <= 1024ll * device_sms()) return false;
     return o.mode == 0 && fits(o.threads_per_tree) && fits(o.pruned_threads_per_tree) && fits(o.small_threads_per_tree);
 }
 

@@ -182,6 +182,20 @@ def test_block_size_of_short_rows(name, first, later, ranged, bare, capfd, monke
         assert np.array_equal(np.diff(off.astype(np.int64)), np.bincount(v[on], minlength=g.n))
 
 
+@pytest.mark.parametrize("per_sm,want", [(0.1, 1024), (1, 1024), (1.5, 512), (2, 512), (3, 256), (4, 256), (5, 128)])
+def test_block_size_at_a_limit_of_trees(per_sm, want, capfd, monkeypatch):
+    """A grid large enough to keep its numbering: few trees in flight take more threads each."""
+    g, rank = case("grid280")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    monkeypatch.setenv("CHL_TRACE", "1")
+    capfd.readouterr()
+    L = chl.build_labels(DG(g), dev(rank), slots=int(per_sm * sms), root_end=3000, small_tree_expansions=1)
+    assert set(re.findall(r" threads (\d+) ", capfd.readouterr().err)) == {str(want)}
+    whole = chl.build_labels(DG(g), dev(rank), root_end=3000)
+    for x, y in zip(whole.to_numpy(), L.to_numpy()):
+        assert np.array_equal(x, y)
+
+
 def test_label_buffer_of_large_road_like_graphs(capfd, monkeypatch):
     """Four grids of 420 x 420 side by side (about 390 labels per vertex): the label
     buffer holds them at once, so that no tree is built twice; the labels are those
