@@ -262,10 +262,12 @@ constexpr uint32_t DIRECT_SMALL_N = 131072;
 // builds at 128 and 1024 threads, random 6-regular, 60,000 vertices (2,500 a
 // round) 822 and 371 ms, random cubic, 30,000 (570) 59 and 52, 3-d mesh, 64,000
 // (390) 199 and 175, 140,000 (470) 599 and 864, randomly numbered grid, 90,000
-// (90) 51 and 111. Local numberings are narrow enough (at most 2% slower than at 1024
-// threads before), and up to DIRECT_SURE_N vertices 128 threads won on every graph
-// tried; the others begin at 1024 threads and leave them where the first trees
-// expand fewer than WIDE_ROUND vertices a round.
+// (90) 51 and 111. Trees of local numberings are narrow enough (random bands of 100,000
+// vertices within the bound, 370 to 560 a round, 97 to 516 ms at 128 threads, 166 to
+// 785 with 1024 and the flat arc pass), and up to DIRECT_SURE_N vertices 128 threads
+// won on every graph tried (random 8-regular, 20,000 vertices, 930 a round: 59 and 62
+// ms; 8,000: 8.7 and 12.7); the others begin at 1024 threads and leave them where the
+// first trees expand fewer than WIDE_ROUND vertices a round.
 constexpr uint32_t DIRECT_SURE_N = 20000;
 constexpr double WIDE_ROUND = 512.0;
 

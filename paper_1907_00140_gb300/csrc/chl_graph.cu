@@ -403,7 +403,8 @@ int grid_for(uint64_t work, int tpb) {
 // together, and the slots' keys stay in the last level cache (grids of 262,000
 // vertices: 143 ms by rank, 127 ms so; 90,000: 33.5 and 32.1; 49,000 and fewer:
 // within 1%, the rank order stays). Scale-free graphs gain more from the rank
-// order, which puts the hubs together.
+// order, which puts the hubs together, and so do random bands twice as wide as the
+// bound (100,000 vertices: 880 ms kept at 256 threads, 667 by rank at 1024).
 // Light-tailed weights only: the block sizes of the other graphs with short rows
 // (choose_params) have no kernels for the caller's numbering.
 static constexpr double LOCAL_GAP = 1.0 / 128;
